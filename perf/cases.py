@@ -206,3 +206,174 @@ def tolerance(case):
     if kind == "attn_f32":
         return {"rel": 2e-4, "max": 0.04}
     return "exact" if kind == "hif8" else {"rel": 6e-7}
+
+
+# ---- the same results in 64 bits, by plain torch ---------------------------------------------------
+
+LOG2E = 1.4426950408889634074
+
+
+def _hif8(x):
+    """Nearest HiF8 value, ties to the larger magnitude: 3 / 2 / 1 mantissa bits for exponents up to 3 / 7 / 15
+    in magnitude, powers of two from 2^-22 to 2^-16, nothing below 2^-23, infinity from 40960 on."""
+    a = x.abs()
+    e = torch.frexp(a.clamp(2.0 ** -22, 65536.0))[1] - 1
+    ae = e.abs()
+    bits = (ae <= 3).int() + (ae <= 7).int() + (ae <= 15).int()
+    step = torch.ldexp(torch.ones_like(a), e - bits)
+    r = torch.floor(a / step + 0.5) * step
+    r = torch.where(a < 2.0 ** -23, 0.0, torch.where(a < 2.0 ** -22, 2.0 ** -22, r))
+    r = torch.where(a >= 40960.0, float("inf"), r)
+    return torch.copysign(r, x)
+
+
+def _w8(t):
+    return _hif8(torch.exp2(_hif8(t)))
+
+
+def _update(s, m, lam, mode, first, whole_tile):
+    """One block of Algorithm 1 (or of Eq. (2) in the other modes): base-2 scores s [..., rows, block] against
+    the running max m [..., rows].  Returns the new max, the weights against it and the max the 8-bit
+    arguments were taken against."""
+    mx = s.amax(-1)
+    if mode != binding.MODE_E2E_HIF8:
+        new = torch.maximum(m, mx)
+        t = s - new[..., None]
+        return new, torch.exp2(t) if mode == binding.MODE_EXACT else _w8(t), new
+    up = torch.maximum(m, torch.ceil(mx))
+    if first:
+        return up, torch.exp2(s - up[..., None]), up
+    r8 = _hif8(mx - m)
+    restart = r8 > lam
+    if whole_tile:
+        restart = restart.any(-1, keepdim=True)
+    new = torch.where(restart, up, m + torch.ceil(r8).clamp_min(0.0))
+    ref = torch.where(restart, up, m)
+    return new, _w8(s - ref[..., None]) * torch.exp2(ref - new)[..., None], ref
+
+
+def _exact_attention(q, k, v, causal, block, lam, mode, b0_last):
+    """q [N,G,S,D], k, v [N,S,D] in 64 bits: N (batch, kv head) pairs of G query heads each.
+    Returns out [N,G,S,D], row max and row sum [N,G,S], restart counts are left out."""
+    N, G, S, D = q.shape
+    n = S // block
+    q = q.view(N, G, n, block, D) * (LOG2E / D ** 0.5)
+    k, v = k.view(N, 1, n, block, D), v.view(N, 1, n, block, D)
+    m = torch.full((N, G, n, block), -float("inf"), dtype=torch.float64, device=q.device)
+    d, o = torch.zeros_like(m), torch.zeros_like(q)
+    above = torch.ones(block, block, dtype=torch.bool, device=q.device).triu(1)
+
+    def step(i0, kt, vt, diag, first):
+        """Query tiles i0 .. against key tiles kt (one for all, or one each); diag: which of them are masked."""
+        s = q[:, :, i0:] @ kt.transpose(-1, -2)
+        if diag is not None:
+            s[:, :, diag] = s[:, :, diag].masked_fill(above, -float("inf"))
+        old = m[:, :, i0:]
+        new, p, _ = _update(s, old, lam, mode, first, True)
+        a = old - new
+        a = torch.where(torch.isinf(old), 0.0, _w8(a) if mode == binding.MODE_EXP2_HIF8 else torch.exp2(a))
+        d[:, :, i0:] = d[:, :, i0:] * a + p.sum(-1)
+        o[:, :, i0:] = o[:, :, i0:] * a[..., None] + p @ vt
+        m[:, :, i0:] = new
+
+    if b0_last and mode == binding.MODE_E2E_HIF8:
+        step(0, k[:, :, :1], v[:, :, :1], 0 if causal else None, True)
+        if n > 1:
+            last = slice(1, n) if causal else slice(n - 1, n)
+            if causal:
+                step(1, k[:, :, last], v[:, :, last], slice(0, n - 1), True)
+            else:
+                step(0, k[:, :, last], v[:, :, last], None, True)
+        for j in range(1, n - 1):
+            step(j + 1 if causal else 0, k[:, :, j:j + 1], v[:, :, j:j + 1], None, False)
+    else:
+        for j in range(n):
+            step(j if causal else 0, k[:, :, j:j + 1], v[:, :, j:j + 1], 0 if causal else None, j == 0)
+    return (o / d[..., None]).view(N, G, S, D), m.view(N, G, S), d.view(N, G, S)
+
+
+def _exact_rows(x, block, codes):
+    """Row softmax: probabilities, or (codes, exponents, row sums) with T rounded once to 32 bits."""
+    rows, cols = x.shape
+    xd = x.double() * (float(torch.tensor(LOG2E, dtype=torch.float32)) if codes else LOG2E)
+    m = torch.full((rows, 1), -float("inf"), dtype=torch.float64, device=x.device)
+    w, refs = torch.empty_like(xd), []
+    for j in range(cols // block):
+        at = slice(j * block, (j + 1) * block)
+        s = xd[:, None, at]
+        if codes and j:
+            s = m[..., None] + (s - m[..., None]).float().double()
+        new, p, ref = _update(s, m, 1, binding.MODE_E2E_HIF8, j == 0, False)
+        if codes and j == 0:
+            p = _w8((s - new[..., None]).float().double())
+        w[:, at] = (p * torch.exp2(new - ref)[..., None])[:, 0]      # against ref
+        refs.append(ref)
+        m = new
+    e = torch.cat(refs, 1) - m
+    w = w.view(rows, -1, block)
+    d = (w.sum(-1) * torch.exp2(e)).sum(-1)
+    if codes:
+        return _codes(w.view(rows, cols)), e.int(), d
+    return w.mul_(torch.exp2(e)[..., None] / d[:, None, None]).view(rows, cols)
+
+
+def _hif8_values():
+    """The 256 values by code: sign, prefix-coded width of the exponent, sign-magnitude exponent, mantissa."""
+    out = []
+    for c in range(128):
+        if c >> 5 == 3:
+            width, mant, rest = 4, 1, c & 31
+        elif c >> 5 == 2:
+            width, mant, rest = 3, 2, c & 31
+        elif c >> 5 == 1:
+            width, mant, rest = 2, 3, c & 31
+        elif c >> 4 == 1:
+            width, mant, rest = 1, 3, c & 15
+        elif c >> 3 == 1:
+            width, mant, rest = 0, 3, c & 7
+        else:
+            out.append(2.0 ** (c - 23) if c else 0.0)
+            continue
+        exp = rest >> mant
+        if width:
+            mag = (1 << (width - 1)) | (exp & ((1 << (width - 1)) - 1))
+            exp = -mag if exp >> (width - 1) else mag
+        out.append((1 + (rest & ((1 << mant) - 1)) / (1 << mant)) * 2.0 ** exp)
+    out[0x6F] = float("inf")
+    neg = [-v for v in out]
+    neg[0] = float("nan")
+    return out + neg
+
+
+def _codes(x):
+    vals = torch.tensor(_hif8_values(), dtype=torch.float64, device=x.device)
+    mags, order = vals[:128].sort()
+    mids = (mags[:-1] + mags[1:]) / 2
+    mids[-1] = 40960.0
+    c = order[torch.searchsorted(mids, x.abs(), right=True)]
+    return torch.where((x < 0) & (c > 0), c + 128, c).to(torch.uint8)
+
+
+def exact(case, seed):
+    kind = case["kind"]
+    state = prepare(case, seed)
+    if kind in ("rows", "codes"):
+        return _exact_rows(state["x"], case["block_k"], kind == "codes")
+    if kind == "hif8":
+        vals = torch.tensor(_hif8_values(), dtype=torch.float64, device="cuda")
+        t = _codes(state["x"].double())
+        p = _codes(torch.exp2(vals))[t.long()]
+        return t, p, vals[p.long()]
+    B, H, Hkv, S, D = (case[n] for n in ("B", "H", "Hkv", "S", "D"))
+    q, k, v = state["q"], state["k"], state["v"]
+    if kind == "attn_fp8":
+        q = (q.view(torch.float8_e4m3fn).float().view(B, H, -1, 128, D) * state["q_scale"][..., None, None]).view(B, H, S, D)
+        k = (k.view(torch.float8_e4m3fn).float().view(B, Hkv, -1, 128, D) * state["k_scale"][..., None, None]).view(B, Hkv, S, D)
+    block, G = case.get("block", 128), H // Hkv
+    q, k, v = q.reshape(B * Hkv, G, S, D), k.reshape(B * Hkv, S, D), v.reshape(B * Hkv, S, D)
+    part = max(1, (1 << 27) // (G * S * block))             # (batch, kv head) pairs at a time
+    got = [_exact_attention(q[i:i + part].double(), k[i:i + part].double(), v[i:i + part].double(), case["causal"],
+                            block, case.get("lam", 1), case.get("mode", binding.MODE_E2E_HIF8), case.get("b0_last", False))
+           for i in range(0, B * Hkv, part)]
+    out, m, d = (torch.cat([g[i] for g in got]).view(B, H, S, *([D] if i == 0 else [])) for i in range(3))
+    return [out, out, m, d, None] if kind == "attn_ex" else out
