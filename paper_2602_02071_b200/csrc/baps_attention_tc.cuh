@@ -550,13 +550,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
         {
             float4 *rep = reinterpret_cast<float4 *>(smem + L::kLutRepOff);
             for (int e = tid; e < kLutRepEntries; e += kTcSoftmaxWarps * 32) {
-                const float w = (e < 16) ? 1.f : g_w0_table[e - 16];
+                const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
                 const float4 w4 = make_float4(w, w, w, w);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) rep[e * 8 + i] = w4;
             }
             float *full = reinterpret_cast<float *>(smem + L::kLutFullOff);
-            for (int i = tid; i < kLutN; i += kTcSoftmaxWarps * 32) full[i] = g_w0_table[i];
+            for (int i = tid; i < kLutN; i += kTcSoftmaxWarps * 32) full[i] = g_w0.v[i];
             named_bar_sync(6, kTcSoftmaxWarps * 32);
         }
         const int q4 = warp & 3;                 // TMEM lane quarter: rows 32 q4 .. 32 q4 + 31
@@ -858,8 +858,6 @@ static inline baps_status attention_tc_launch(const void *q, const void *k, cons
                                        const float *q_scale = nullptr, const float *k_scale = nullptr)
 {
     const bool qk8 = q_scale != nullptr;               // Q, K are E4M3 codes with per-tile scales
-    const baps_status ts = ensure_w0_table(stream);
-    if (ts != BAPS_OK) return ts;
     CUtensorMap mq, mk, mv;
     if (qk8) {
         if (!make_tmap_u8_rows(&mq, q, (uint64_t)B * H * S, (uint64_t)D, 128) ||

@@ -123,17 +123,6 @@ constexpr int kLutPosHi = ((127 + 2) << 4) - 1;             // last key below +4
 constexpr int kLutPosN = kLutPosHi - kLutPosLo + 1;
 constexpr int kLutN = kLutNegN + kLutPosN;                  // 177 + 128 entries
 
-// Entry i of the table (device-side build; 2^t in double so that no entry depends on the
-// accuracy of the hardware exponential).
-__device__ __forceinline__ float w0_table_entry(int i)
-{
-    uint32_t key;
-    if (i < kLutNegN) key = (uint32_t)(kLutNegLo + i);
-    else key = (uint32_t)(kLutPosLo + (i - kLutNegN));
-    const float u = __uint_as_float(key << 19);
-    return hif8_exp2_value(hif8_round(u));
-}
-
 // Index of u into the table.
 __device__ __forceinline__ int w0_index(float u)
 {

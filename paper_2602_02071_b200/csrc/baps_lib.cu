@@ -39,18 +39,14 @@ baps_status set_smem(K kernel, size_t bytes)
     return BAPS_OK;
 }
 
-baps_status attention_f32_launch(const AttnF32Params &p, int bq, int bk, cudaStream_t st)
+template <int BLK>
+baps_status attention_f32_launch(const AttnF32Params &p, cudaStream_t st)
 {
-    dim3 grid(p.S / bq, p.H, p.B);
-    if (bq == 64) {
-        const size_t sm = attention_f32_smem<64, 64>();
-        if (set_smem(attention_f32_kernel<64, 64>, sm) != BAPS_OK) return BAPS_ERR_CUDA;
-        attention_f32_kernel<64, 64><<<grid, kAfThreads, sm, st>>>(p);
-    } else {
-        const size_t sm = attention_f32_smem<128, 128>();
-        if (set_smem(attention_f32_kernel<128, 128>, sm) != BAPS_OK) return BAPS_ERR_CUDA;
-        attention_f32_kernel<128, 128><<<grid, kAfThreads, sm, st>>>(p);
-    }
+    using L = AfLayout<BLK>;
+    const size_t sm = sizeof(float) * (size_t)L(p.D).total;
+    if (set_smem(attention_f32_kernel<BLK>, sm) != BAPS_OK) return BAPS_ERR_CUDA;
+    const dim3 grid((unsigned)(p.S / BLK) * kAfCluster, p.H, p.B);
+    attention_f32_kernel<BLK><<<grid, L::THREADS, sm, st>>>(p);
     return launch_status();
 }
 
@@ -294,7 +290,7 @@ baps_status baps_attention_fwd_ex(const void *q, const void *k, const void *v, v
         p.restarts = s.restarts;
         p.B = B; p.H = H; p.Hkv = Hkv; p.S = S; p.D = D; p.causal = causal ? 1 : 0;
         p.lambda = o.lambda; p.mode = o.mode; p.c = c; p.b0_last = o.b0_last ? 1 : 0;
-        return attention_f32_launch(p, block_q, block_k, as_stream(stream));
+        return block_q == 64 ? attention_f32_launch<64>(p, as_stream(stream)) : attention_f32_launch<128>(p, as_stream(stream));
     }
     if (dtype == BAPS_DTYPE_BF16) {
         if (block_q != 128 || block_k != 128) return BAPS_ERR_UNSUPPORTED;

@@ -187,9 +187,9 @@ softmax_rows_generic_kernel(const float *__restrict__ logits, float *__restrict_
     const int nb = cols / BK;
     const int nchunks = cols / 128;            // a warp step covers 128 elements
 
-    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = g_w0_table[i];
+    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = g_w0.v[i];
     for (int e = tid; FAST && e < 16 + kLutNegN; e += THREADS) {
-        const float w = (e < 16) ? 1.f : g_w0_table[e - 16];
+        const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
         const float4 w4 = make_float4(w, w, w, w);
 #pragma unroll
         for (int i = 0; i < 8; ++i) reinterpret_cast<float4 *>(s_rep)[e * 8 + i] = w4;
@@ -316,9 +316,9 @@ struct RowsOut {
 template <bool CODES, int NTHREADS>
 __device__ __forceinline__ void fill_tables(uint32_t *s_lut, uint32_t *s_rep, int t)
 {
-    for (int i = t; i < kLutN; i += NTHREADS) s_lut[i] = CODES ? w0_word(g_w0_table[i]) : __float_as_uint(g_w0_table[i]);
+    for (int i = t; i < kLutN; i += NTHREADS) s_lut[i] = CODES ? w0_word(g_w0.v[i]) : __float_as_uint(g_w0.v[i]);
     for (int e = t; e < 16 + kLutNegN; e += NTHREADS) {
-        const float w = (e < 16) ? 1.f : g_w0_table[e - 16];
+        const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
         const uint32_t u = CODES ? w0_word(w) : __float_as_uint(w);
         const uint4 u4 = make_uint4(u, u, u, u);
 #pragma unroll
@@ -899,9 +899,9 @@ softmax_rows_codes_generic_kernel(const float *__restrict__ logits, uint8_t *__r
     constexpr int kWarps = THREADS / 32;
     constexpr int LPB = BK / 4, BPW = 32 / LPB;
     const int nb = cols / BK, nchunks = cols / 128;
-    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = w0_word(g_w0_table[i]);
+    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = w0_word(g_w0.v[i]);
     for (int e = tid; FAST && e < 16 + kLutNegN; e += THREADS) {
-        const uint32_t u = w0_word((e < 16) ? 1.f : g_w0_table[e - 16]);
+        const uint32_t u = w0_word((e < 16) ? 1.f : g_w0.v[e - 16]);
         const uint4 u4 = make_uint4(u, u, u, u);
 #pragma unroll
         for (int i = 0; i < 8; ++i) reinterpret_cast<uint4 *>(s_rep)[e * 8 + i] = u4;
@@ -970,8 +970,6 @@ template <int BK>
 inline baps_status softmax_rows_codes_dispatch(const float *logits, uint8_t *codes, int32_t *block_exp, float *row_d,
                                                int64_t rows, int cols, int lambda, int num_sms, cudaStream_t st)
 {
-    const baps_status ts = ensure_w0_table(st);
-    if (ts != BAPS_OK) return ts;
     auto grid_for = [&](int ctas_per_sm) {
         const int64_t cap = (int64_t)num_sms * ctas_per_sm;
         return (int)(rows < cap ? rows : cap);
@@ -1016,8 +1014,6 @@ template <int BK>
 inline baps_status softmax_rows_dispatch(const float *logits, float *probs, int64_t rows, int cols, int lambda,
                                   int num_sms, cudaStream_t st)
 {
-    const baps_status ts = ensure_w0_table(st);
-    if (ts != BAPS_OK) return ts;
     auto grid_for = [&](int ctas_per_sm) {
         const int64_t cap = (int64_t)num_sms * ctas_per_sm;
         return (int)(rows < cap ? rows : cap);

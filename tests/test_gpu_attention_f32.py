@@ -75,3 +75,20 @@ def test_f32_kernel_b0_first_and_last(causal, bq, S):
     st, ref = _run(w, b0_last=True)
     gate_attention(st.out_f32.cpu().numpy(), ref, what=f"f32 b0 first+last causal={causal} bq={bq} S={S}")
     assert np.array_equal(st.restarts.cpu().numpy().ravel(), ref.restarts)
+
+
+@pytest.mark.parametrize("bq,S", [(64, 64), (64, 192), (128, 256)])
+@pytest.mark.parametrize("D", [4, 20, 32, 80, 100, 128])
+def test_f32_kernel_head_sizes(D, bq, S):
+    """Head sizes that leave the 16-column steps of the score products and the key groups of the value
+    product ragged; every row is compared (the tile is shared by eight CTAs).  A masked key must not reach the
+    output even where its V is infinite."""
+    w = workloads.AttnWorkload("t", 1, 4, 2, S, D, True, bq, bq, dtype="f32", seed=D + S)
+    st, ref = _run(w)
+    gate_attention(st.out_f32.cpu().numpy(), ref, what=f"f32 D={D} bq={bq} S={S}")
+    assert np.array_equal(st.restarts.cpu().numpy().ravel(), ref.restarts)
+    assert np.allclose(st.row_d.cpu().numpy().reshape(ref.row_d.shape), ref.row_d, rtol=1e-4)
+    q, k, v = (t.cuda() for t in workloads.make_qkv(w))
+    v[:, :, -1] = float("inf")                  # only the last query sees the last key
+    out = binding.baps_attention_fwd_f32(q, k, v, causal=True, block_q=bq, block_k=bq)
+    assert torch.equal(out[:, :, :-1], st.out_f32[:, :, :-1])
