@@ -7,13 +7,15 @@
 //           at blocks whose maximum exceeds it, so the warp tests 32 blocks per ballot;
 //   pass 2  form the 8-bit weights, reduce d;
 //   pass 3  write p = w * 2^(m_block - m_final) / d.
-// Rows of 1K columns are handled by one warp each (softmax_rows_warp_kernel), rows of 2K, 4K and 8K
-// columns by groups of threads that share a CTA and its tables (softmax_rows_group_kernel), rows of 16K
-// and 32K by one CTA each, fed through a shared-memory ring by bulk asynchronous copies so that the read
-// of the next row overlaps the passes over the current one, rows of 64K by one CTA that keeps half the row
-// in registers and half in the shared-memory pieces it arrived in.  In all of these the row stays on chip
-// between the passes, so HBM traffic is exactly one read and one write of the row (8 bytes per element).  Other lengths use the generic variant, which re-reads
-// the row from L2 in passes 2 and 3.
+// Rows of up to 1K columns are handled by one warp each (softmax_rows_warp_kernel), rows of up to 8K columns
+// by groups of threads that share a CTA and its tables (softmax_rows_group_kernel), rows of up to 32K by one
+// CTA each, fed through a shared-memory ring by bulk asynchronous copies so that the read of the next row
+// overlaps the passes over the current one, longer rows by one CTA that keeps half the row in registers and
+// half in the shared-memory pieces it arrived in.  In all of these the row stays on chip between the passes,
+// so HBM traffic is exactly one read and one write of the row (8 bytes per element).  FULL instances know
+// the row length (the largest of their range, a power of two) at compile time; the others take it as an
+// argument and leave out the 128-column chunks past the end.  (Measured on 2^27 logits against a variant that
+// re-read every row twice from L2: 640 columns 720 -> 189 us, 3200 397 -> 216, 12800 304 -> 219, 49152 280 -> 249.)
 // Blocks whose T are all <= 0 (nearly all of them) take the weights from a bank-replicated table keyed
 // by the top bits of -T * 2^-120, as the fused attention kernel does.  What a block's weights need --
 // the max its T are taken against, the power of two that moves them to the final max, which table --
@@ -25,8 +27,6 @@
 #include "baps_sm100.cuh"
 
 namespace baps {
-
-constexpr int kSrMaxBlocks = 1024;     // 65536 / 64
 
 // Max bookkeeping of Algorithm 1 for one block of a single row: given the running max m
 // (integer valued, or -inf before block 0) and the block's largest logit xmax (base-2 score
@@ -85,7 +85,6 @@ __device__ __forceinline__ BlockParams block_params(float mb, float bm, bool fir
 // Weights of one 16-byte vector of a block, already moved to the final max.  any_pos: some block of
 // this warp-wide vector holds a positive T (warp-uniform for BK = 128), in which case the whole vector
 // takes the full table.
-template <bool FAST>
 __device__ __forceinline__ float4 block_weights(const float4 &x, float mref, float scale, int kind, bool any_pos,
                                                 const float *s_rep, const float *s_lut, int lane)
 {
@@ -93,7 +92,7 @@ __device__ __forceinline__ float4 block_weights(const float4 &x, float mref, flo
     if (kind == 0) {
         w.x = exp2f(fmaf(x.x, kLog2e, -mref)); w.y = exp2f(fmaf(x.y, kLog2e, -mref));
         w.z = exp2f(fmaf(x.z, kLog2e, -mref)); w.w = exp2f(fmaf(x.w, kLog2e, -mref));
-    } else if (FAST && !any_pos) {
+    } else if (!any_pos) {
         // x = -T * 2^-120 by one fused multiply-add with flush-to-zero (|T| < 2^-6 becomes +0, weight
         // 1), the top bits of x select the entry (everything from |T| >= 32 on is the entry 0)
         const float cn = -kLog2e * 7.52316384526264e-37f, mn = mref * 7.52316384526264e-37f;   // 2^-120
@@ -121,21 +120,20 @@ __device__ __forceinline__ int pack_kind(int kind)
     return kind | (slow << 2);
 }
 
-// The scan of Algorithm 1's max bookkeeping over the NB block maxima of one row, by one warp: writes the
+// The scan of Algorithm 1's max bookkeeping over the nb block maxima of one row, by one warp: writes the
 // running max before every block and the final max.  The state is one integer per row and only changes at
 // blocks whose maximum exceeds it, so the warp tests 32 blocks per ballot.  (The loop over the groups of
 // 32 blocks is kept rolled: unrolled, with the inner loop and the update inlined four or more times, the
 // same kernel ran 20 % slower.)
-template <int NB>
-__device__ __forceinline__ void scan_blocks(const float *s_bmax, float *s_mbefore, float *s_mfinal, int lambda, int lane)
+__device__ __forceinline__ void scan_blocks(int nb, const float *s_bmax, float *s_mbefore, float *s_mfinal, int lambda, int lane)
 {
     bool rs; float dl;
     float m = row_block_update(-INFINITY, s_bmax[0], true, lambda, &rs, &dl);
     if (lane == 0) s_mbefore[0] = -INFINITY;
 #pragma unroll 1
-    for (int base = 1; base < NB; base += 32) {
+    for (int base = 1; base < nb; base += 32) {
         const int j = base + lane;
-        const bool valid = j < NB;
+        const bool valid = j < nb;
         const float mj = valid ? s_bmax[j] : -INFINITY;
         bool pending = valid;
         while (true) {
@@ -164,105 +162,6 @@ __device__ __forceinline__ void bulk_load_row(uint32_t dst, const float *src, ui
     }
 }
 
-// Any row length that is a multiple of 128 (the lengths without a kernel of their own): one CTA per row
-// at a time, the row is read three times -- from HBM for the block maxima, then again (from L2) for the
-// sum of the weights and for the output.  BK: block size of Algorithm 1 along the row (64 or 128).
-// FAST: blocks without a positive T use the bank-replicated table (25 KB of shared memory).
-template <int BK, int THREADS, bool FAST>
-__global__ void __launch_bounds__(THREADS)
-softmax_rows_generic_kernel(const float *__restrict__ logits, float *__restrict__ probs, int64_t rows,
-                            int cols, int lambda)
-{
-    __shared__ float s_bmax[kSrMaxBlocks];     // block maxima of the logits
-    __shared__ float s_mbefore[kSrMaxBlocks];  // running max before each block (m~)
-    __shared__ float s_lut[kLutN];
-    __shared__ __align__(16) float s_rep[FAST ? (16 + kLutNegN) * 32 : 32];
-    __shared__ float s_red[THREADS / 32];
-    __shared__ float s_mfinal;
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int kWarps = THREADS / 32;
-    constexpr int LPB = BK / 4;                // lanes per block (float4 per lane)
-    constexpr int BPW = 32 / LPB;              // blocks per warp step (1 for 128, 2 for 64)
-    const int nb = cols / BK;
-    const int nchunks = cols / 128;            // a warp step covers 128 elements
-
-    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = g_w0.v[i];
-    for (int e = tid; FAST && e < 16 + kLutNegN; e += THREADS) {
-        const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
-        const float4 w4 = make_float4(w, w, w, w);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) reinterpret_cast<float4 *>(s_rep)[e * 8 + i] = w4;
-    }
-    __syncthreads();
-
-    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-        const float4 *x4 = reinterpret_cast<const float4 *>(logits + row * cols);
-        float4 *p4 = reinterpret_cast<float4 *>(probs + row * cols);
-        // ---- pass 1: block maxima (the only HBM read of the row) ----------------------------------------
-        for (int ch = warp; ch < nchunks; ch += kWarps) {
-            const float4 x = __ldg(x4 + ch * 32 + lane);
-            float mx = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
-            mx = lanes_max<LPB>(mx);
-            if ((lane % LPB) == 0) s_bmax[ch * BPW + lane / LPB] = mx;
-        }
-        __syncthreads();
-        // ---- scan over the blocks (warp 0) ---------------------------------------------------------------
-        if (warp == 0) {
-            bool rs; float dl;
-            float m = row_block_update(-INFINITY, s_bmax[0], true, lambda, &rs, &dl);
-            if (lane == 0) s_mbefore[0] = -INFINITY;
-            for (int base = 1; base < nb; base += 32) {
-                const int j = base + lane;
-                const bool valid = j < nb;
-                const float mj = valid ? s_bmax[j] : -INFINITY;
-                bool pending = valid;
-                while (true) {
-                    // HiF8(T) > 0  <=>  T >= 2^-23 (smaller magnitudes round to zero)
-                    const bool pred = pending && fmaf(mj, kLog2e, -m) >= 1.1920928955078125e-07f;
-                    const unsigned b = __ballot_sync(0xffffffffu, pred);
-                    if (b == 0u) { if (pending) s_mbefore[j] = m; break; }
-                    const int l = __ffs(b) - 1;
-                    if (pending && lane <= l) { s_mbefore[j] = m; pending = false; }
-                    const float ml = __shfl_sync(0xffffffffu, mj, l);
-                    m = row_block_update(m, ml, false, lambda, &rs, &dl);
-                }
-            }
-            if (lane == 0) s_mfinal = m;
-        }
-        __syncthreads();
-        const float mfinal = s_mfinal;
-        // weights of one 16-byte vector, already moved to the final max
-        auto weights = [&](const float4 &x, int ch) {
-            const int j = ch * BPW + lane / LPB;
-            const BlockParams bp = block_params(s_mbefore[j], s_bmax[j], j == 0, lambda, mfinal);
-            // some lane of the warp holds a block with a positive T: voted by the whole warp
-            const bool any_pos = __any_sync(0xffffffffu, bp.kind == 2);
-            return block_weights<FAST>(x, bp.mref, bp.scale, bp.kind, any_pos, s_rep, s_lut, lane);
-        };
-        // ---- pass 2: the sum of the weights ----------------------------------------------------------------
-        float dsum = 0.f;
-        for (int ch = warp; ch < nchunks; ch += kWarps) {
-            const float4 w = weights(__ldg(x4 + ch * 32 + lane), ch);
-            dsum += (w.x + w.y) + (w.z + w.w);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-        if (lane == 0) s_red[warp] = dsum;
-        __syncthreads();
-        float t = 0.f;                          // every thread adds the partial sums itself, in the same order
-#pragma unroll
-        for (int i = 0; i < kWarps; ++i) t += s_red[i];
-        const float dinv = 1.f / t;
-        // ---- pass 3: p = w * 2^(m_block - m_final) / d -----------------------------------------------------
-        for (int ch = warp; ch < nchunks; ch += kWarps) {
-            const float4 w = weights(__ldg(x4 + ch * 32 + lane), ch);
-            __stcs(p4 + ch * 32 + lane, make_float4(w.x * dinv, w.y * dinv, w.z * dinv, w.w * dinv));
-        }
-        __syncthreads();   // s_bmax / s_mbefore / s_red are reused by the next row
-    }
-}
-
 // Table words of the 8-bit-output kernels: the fp32 pattern of w0(T) with its HiF8 code in the low byte.
 __device__ __forceinline__ uint32_t w0_word(float w) { return __float_as_uint(w) | (uint32_t)hif8_pack(w); }
 
@@ -282,12 +181,11 @@ __device__ __forceinline__ CodesBlockParams codes_block_params(float mb, float b
 }
 
 // Table words of one 16-byte vector.
-template <bool FAST>
 __device__ __forceinline__ uint4 block_words(const float4 &x, float mref, bool any_pos, const uint32_t *s_rep,
                                              const uint32_t *s_lut, int lane)
 {
     uint4 e;
-    if (FAST && !any_pos) {
+    if (!any_pos) {
         const float cn = -kLog2e * 7.52316384526264e-37f, mn = mref * 7.52316384526264e-37f;   // 2^-120
         auto fast = [&](float xv) {
             float t;
@@ -341,19 +239,20 @@ __device__ __forceinline__ float emit_codes(uint32_t *dst, const uint4 &e, float
 // thread issues as soon as the current row sits in registers, i.e. after the first barrier of the row:
 // the HBM read of the next row overlaps the scan, the weights and the write of the current one.
 // Three barriers per row.  CODES: 8-bit output.
-template <int BK, int THREADS, bool CODES, bool REDUX = true>
+template <int BK, int THREADS, bool CODES, bool REDUX = true, bool FULL = true>
 __global__ void __launch_bounds__(THREADS, 2048 / THREADS / 2)
-softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda)
+softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda, int cols_)
 {
-    constexpr int NV = 8, kWarps = THREADS / 32, cols = NV * THREADS * 4;
-    constexpr int LPB = BK / 4, BPW = 32 / LPB, nb = cols / BK;
-    constexpr uint32_t row_bytes = (uint32_t)cols * 4u;
+    constexpr int NV = 8, kWarps = THREADS / 32, kCols = NV * THREADS * 4;
+    constexpr int LPB = BK / 4, BPW = 32 / LPB;
+    const int cols = FULL ? kCols : cols_, nch = cols / 128, nb = cols / BK;
+    const uint32_t row_bytes = (uint32_t)cols * 4u;
     static_assert(NV * BPW <= 32, "one block per lane");
     extern __shared__ __align__(128) uint8_t sr_ring[];          // one row
     __shared__ __align__(8) uint64_t s_full;
     __shared__ int s_abort;
-    __shared__ float s_bmax[nb];
-    __shared__ float s_mbefore[nb];
+    __shared__ float s_bmax[kCols / BK];
+    __shared__ float s_mbefore[kCols / BK];
     __shared__ uint32_t s_lut[kLutN];
     __shared__ __align__(16) uint32_t s_rep[(16 + kLutNegN) * 32];
     __shared__ float s_red[kWarps];
@@ -382,10 +281,12 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
         {
             const float4 *ring4 = reinterpret_cast<const float4 *>(sr_ring);
 #pragma unroll
-            for (int k = 0; k < NV; ++k) v[k] = ring4[(warp + k * kWarps) * 32 + lane];
+            for (int k = 0; k < NV; ++k)
+                if (FULL || warp + k * kWarps < nch) v[k] = ring4[(warp + k * kWarps) * 32 + lane];
         }
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
+            if (!FULL && warp + k * kWarps >= nch) break;
             float mx = fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w));
             mx = lanes_max<LPB, REDUX>(mx);
             if ((lane % LPB) == 0) s_bmax[(warp + k * kWarps) * BPW + lane / LPB] = mx;
@@ -400,7 +301,7 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
             }
         }
         // ---- scan over the blocks (warp 0) ---------------------------------------------------------------
-        if (warp == 0) scan_blocks<nb>(s_bmax, s_mbefore, &s_mfinal, lambda, lane);
+        if (warp == 0) scan_blocks(nb, s_bmax, s_mbefore, &s_mfinal, lambda, lane);
         __syncthreads();
         const float mfinal = s_mfinal;
         const int jmine = (warp + (lane / BPW) * kWarps) * BPW + lane % BPW;      // the block whose parameters I work out
@@ -409,31 +310,33 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
             // ---- pass 2: codes, block exponents, the sum of the decoded weights ---------------------------
             uint32_t *c4 = reinterpret_cast<uint32_t *>(out.codes + row * cols);
             CodesBlockParams bp = {0.f, 0, 1, 0.f};
-            if (lane < NV * BPW) {
+            if (lane < NV * BPW && (FULL || jmine < nb)) {
                 bp = codes_block_params(s_mbefore[jmine], s_bmax[jmine], jmine == 0, lambda, mfinal);
                 out.block_exp[row * nb + jmine] = bp.bexp;
             }
             const int kindp = pack_kind<BPW>(bp.kind);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
+                if (!FULL && warp + k * kWarps >= nch) break;
                 const int src = k * BPW + lane / LPB;
                 const float mref = __shfl_sync(0xffffffffu, bp.mref, src);
                 const float be = __shfl_sync(0xffffffffu, bp.scale, src);
                 const int kp = __shfl_sync(0xffffffffu, kindp, src);
                 dsum += emit_codes(c4 + (warp + k * kWarps) * 32 + lane,
-                                   block_words<true>(v[k], mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
+                                   block_words(v[k], mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
             }
         } else {
             // ---- pass 2: weights (already moved to the final max) and their sum ---------------------------
             BlockParams bp = {0.f, 0.f, 1};
-            if (lane < NV * BPW) bp = block_params(s_mbefore[jmine], s_bmax[jmine], jmine == 0, lambda, mfinal);
+            if (lane < NV * BPW && (FULL || jmine < nb)) bp = block_params(s_mbefore[jmine], s_bmax[jmine], jmine == 0, lambda, mfinal);
             const int kindp = pack_kind<BPW>(bp.kind);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
+                if (!FULL && warp + k * kWarps >= nch) break;
                 const int src = k * BPW + lane / LPB;
                 const float mref = __shfl_sync(0xffffffffu, bp.mref, src), scale = __shfl_sync(0xffffffffu, bp.scale, src);
                 const int kp = __shfl_sync(0xffffffffu, kindp, src);
-                v[k] = block_weights<true>(v[k], mref, scale, kp & 3, (kp & 4) != 0, reinterpret_cast<const float *>(s_rep),
+                v[k] = block_weights(v[k], mref, scale, kp & 3, (kp & 4) != 0, reinterpret_cast<const float *>(s_rep),
                                            reinterpret_cast<const float *>(s_lut), lane);
                 dsum += (v[k].x + v[k].y) + (v[k].z + v[k].w);
             }
@@ -459,8 +362,9 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
             float4 *p4 = reinterpret_cast<float4 *>(out.probs + row * cols);
 #pragma unroll
             for (int k = 0; k < NV; ++k)
-                __stcs(p4 + (warp + k * kWarps) * 32 + lane,
-                       make_float4(v[k].x * dinv, v[k].y * dinv, v[k].z * dinv, v[k].w * dinv));
+                if (FULL || warp + k * kWarps < nch)
+                    __stcs(p4 + (warp + k * kWarps) * 32 + lane,
+                           make_float4(v[k].x * dinv, v[k].y * dinv, v[k].z * dinv, v[k].w * dinv));
         }
         // (no barrier here: what the next row writes first, s_bmax, was last read before the third barrier
         // above; s_mbefore, s_mfinal and s_red are written behind the next row's first and second barrier,
@@ -478,19 +382,23 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
 // next row's quarter 0 once quarter 1 does; the piece of quarter 2 takes the next row's quarter 2 when the
 // output pass is through with it, likewise quarter 3 -- so of the next row only quarter 1 is waited for in
 // the open.  Seven barriers per row.
-template <int BK, bool CODES>
+template <int BK, bool CODES, bool FULL = true>
 __global__ void __launch_bounds__(1024, 1)
-softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda)
+softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda, int cols_)
 {
-    constexpr int THREADS = 1024, NQ = 4, kWarps = THREADS / 32, kQuarter = NQ * THREADS * 4, cols = 4 * kQuarter;
-    constexpr int LPB = BK / 4, BPW = 32 / LPB, nbq = kQuarter / BK, nb = 4 * nbq;
+    constexpr int THREADS = 1024, NQ = 4, kWarps = THREADS / 32, kQuarter = NQ * THREADS * 4, kCols = 4 * kQuarter;
+    constexpr int LPB = BK / 4, BPW = 32 / LPB, nbq = kQuarter / BK;
+    const int cols = FULL ? kCols : cols_, nb = cols / BK;       // more than half of kCols
+    // 128-column chunks of quarters 2 and 3 (the first two are whole)
+    const int nch2 = FULL ? kQuarter / 128 : min(cols - 2 * kQuarter, kQuarter) / 128;
+    const int nch3 = FULL ? kQuarter / 128 : max(cols - 3 * kQuarter, 0) / 128;
     constexpr uint32_t q_bytes = (uint32_t)kQuarter * 4u;
     static_assert(NQ * BPW <= 32, "one block per lane and quarter");
     extern __shared__ __align__(128) uint8_t sr_ring[];          // three pieces of one quarter row each
     __shared__ __align__(8) uint64_t s_full[3];
     __shared__ int s_abort;
-    __shared__ float s_bmax[nb];
-    __shared__ float s_mbefore[nb];
+    __shared__ float s_bmax[kCols / BK];
+    __shared__ float s_mbefore[kCols / BK];
     __shared__ uint32_t s_lut[kLutN];
     __shared__ __align__(16) uint32_t s_rep[(16 + kLutNegN) * 32];
     __shared__ float s_red[kWarps];
@@ -506,9 +414,11 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
     __syncthreads();
     // one thread: piece `pc` takes quarter `q` of row `r`
     auto request = [&](int pc, int64_t r, int q) {
+        const uint32_t bytes = FULL || q < 2 ? q_bytes : (uint32_t)(q == 2 ? nch2 : nch3) * 512u;
+        if (bytes == 0u) return;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        sm100::mbar_arrive_expect_tx(sm100::smem_u32(&s_full[pc]), q_bytes);
-        bulk_load_row(sm100::smem_u32(sr_ring) + (uint32_t)pc * q_bytes, logits + r * cols + (int64_t)q * kQuarter, q_bytes,
+        sm100::mbar_arrive_expect_tx(sm100::smem_u32(&s_full[pc]), bytes);
+        bulk_load_row(sm100::smem_u32(sr_ring) + (uint32_t)pc * q_bytes, logits + r * cols + (int64_t)q * kQuarter, bytes,
                       sm100::smem_u32(&s_full[pc]));
     };
     if (tid == 0 && (int64_t)blockIdx.x < rows) {
@@ -531,6 +441,8 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
         mx = lanes_max<LPB>(mx);
         if ((lane % LPB) == 0) s_bmax[j0 + lane / LPB] = mx;
     };
+    // does quarter q hold my warp's vector k?
+    auto has = [&](int q, int k) { return FULL || q < 2 || warp + k * kWarps < (q == 2 ? nch2 : nch3); };
     const int vi0 = warp * 32 + lane;           // my vector k of a quarter is number vi0 + k * THREADS of it
 
     for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
@@ -554,12 +466,14 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
         // ---- quarters 2 and 3: stay in their pieces; block maxima -------------------------------------------
         wait_piece(1, ph1, 0x422);
 #pragma unroll
-        for (int k = 0; k < NQ; ++k) block_max(piece[1][vi0 + k * THREADS], 2 * nbq + (warp + k * kWarps) * BPW);
-        wait_piece(2, ph2, 0x423);
+        for (int k = 0; k < NQ; ++k)
+            if (has(2, k)) block_max(piece[1][vi0 + k * THREADS], 2 * nbq + (warp + k * kWarps) * BPW);
+        if (FULL || nch3 > 0) wait_piece(2, ph2, 0x423);
 #pragma unroll
-        for (int k = 0; k < NQ; ++k) block_max(piece[2][vi0 + k * THREADS], 3 * nbq + (warp + k * kWarps) * BPW);
+        for (int k = 0; k < NQ; ++k)
+            if (has(3, k)) block_max(piece[2][vi0 + k * THREADS], 3 * nbq + (warp + k * kWarps) * BPW);
         __syncthreads();
-        if (warp == 0) scan_blocks<nb>(s_bmax, s_mbefore, &s_mfinal, lambda, lane);
+        if (warp == 0) scan_blocks(nb, s_bmax, s_mbefore, &s_mfinal, lambda, lane);
         __syncthreads();
         const float mfinal = s_mfinal;
         // the block of quarter qq whose parameters my lane works out (lane < NQ * BPW)
@@ -570,21 +484,22 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
 #pragma unroll
             for (int qq = 0; qq < 4; ++qq) {
                 CodesBlockParams bp = {0.f, 0, 1, 0.f};
-                if (lane < NQ * BPW) {
-                    const int j = qq * nbq + jl;
+                const int j = qq * nbq + jl;
+                if (lane < NQ * BPW && (FULL || j < nb)) {
                     bp = codes_block_params(s_mbefore[j], s_bmax[j], j == 0, lambda, mfinal);
                     out.block_exp[row * nb + j] = bp.bexp;
                 }
                 const int kindp = pack_kind<BPW>(bp.kind);
 #pragma unroll
                 for (int k = 0; k < NQ; ++k) {
+                    if (!has(qq, k)) break;
                     const int src = k * BPW + lane / LPB;
                     const float mref = __shfl_sync(0xffffffffu, bp.mref, src);
                     const float be = __shfl_sync(0xffffffffu, bp.scale, src);
-                const int kp = __shfl_sync(0xffffffffu, kindp, src);
+                    const int kp = __shfl_sync(0xffffffffu, kindp, src);
                     const float4 x = qq < 2 ? v[qq * NQ + k] : piece[qq - 1][vi0 + k * THREADS];
                     dsum += emit_codes(c4 + qq * (kQuarter / 4) + vi0 + k * THREADS,
-                                       block_words<true>(x, mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
+                                       block_words(x, mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
                 }
             }
 #pragma unroll
@@ -605,8 +520,8 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
 #pragma unroll
             for (int qq = 0; qq < 4; ++qq) {
                 bp[qq] = {0.f, 0.f, 1};
-                if (lane < NQ * BPW) {
-                    const int j = qq * nbq + jl;
+                const int j = qq * nbq + jl;
+                if (lane < NQ * BPW && (FULL || j < nb)) {
                     bp[qq] = block_params(s_mbefore[j], s_bmax[j], j == 0, lambda, mfinal);
                 }
                 kindp[qq] = pack_kind<BPW>(bp[qq].kind);
@@ -615,7 +530,7 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
                 const int src = k * BPW + lane / LPB;
                 const float mref = __shfl_sync(0xffffffffu, bp[qq].mref, src), scale = __shfl_sync(0xffffffffu, bp[qq].scale, src);
                 const int kp = __shfl_sync(0xffffffffu, kindp[qq], src);
-                return block_weights<true>(x, mref, scale, kp & 3, (kp & 4) != 0, f_rep, f_lut, lane);
+                return block_weights(x, mref, scale, kp & 3, (kp & 4) != 0, f_rep, f_lut, lane);
             };
             // ---- weights of all four quarters (moved to the final max) and their sum -----------------------
 #pragma unroll
@@ -629,6 +544,7 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
             for (int qq = 2; qq < 4; ++qq)
 #pragma unroll
                 for (int k = 0; k < NQ; ++k) {
+                    if (!has(qq, k)) break;
                     const float4 w = weights(qq, k, piece[qq - 1][vi0 + k * THREADS]);
                     dsum += (w.x + w.y) + (w.z + w.w);
                 }
@@ -649,6 +565,7 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
             for (int qq = 2; qq < 4; ++qq) {
 #pragma unroll
                 for (int k = 0; k < NQ; ++k) {
+                    if (!has(qq, k)) break;
                     const float4 w = weights(qq, k, piece[qq - 1][vi0 + k * THREADS]);
                     __stcs(p4 + qq * (kQuarter / 4) + vi0 + k * THREADS, make_float4(w.x * dinv, w.y * dinv, w.z * dinv, w.w * dinv));
                 }
@@ -665,15 +582,16 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
 // hardware barrier (three per row), so the groups drift freely against each other.  With the tables
 // shared, an SM holds as many rows in flight as its threads allow, where one-row CTAs stop at the six or
 // seven copies of the 25 KB table that fit its shared memory.  CODES: 8-bit output.
-template <int BK, int THREADS, int NV, int GROUPS, bool CODES, bool PF = true, bool REDUX = true>
+template <int BK, int THREADS, int NV, int GROUPS, bool CODES, bool PF = true, bool REDUX = true, bool FULL = true>
 __global__ void __launch_bounds__(THREADS * GROUPS)
-softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda)
+softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda, int cols_)
 {
-    constexpr int cols = NV * THREADS * 4, nb = cols / BK, kWarps = THREADS / 32;
+    constexpr int kCols = NV * THREADS * 4, kWarps = THREADS / 32;
     constexpr int LPB = BK / 4, BPW = 32 / LPB;
+    const int cols = FULL ? kCols : cols_, nch = cols / 128, nb = cols / BK;
     static_assert(GROUPS >= 1 && GROUPS <= 15 && NV * BPW <= 32, "barrier ids 1 .. 15; one block per lane");
-    __shared__ float s_bmax[GROUPS][nb];
-    __shared__ float s_mbefore[GROUPS][nb];
+    __shared__ float s_bmax[GROUPS][kCols / BK];
+    __shared__ float s_mbefore[GROUPS][kCols / BK];
     __shared__ uint32_t s_lut[kLutN];
     __shared__ __align__(16) uint32_t s_rep[(16 + kLutNegN) * 32];
     __shared__ float s_red[GROUPS][kWarps];
@@ -691,7 +609,8 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
     if (PF && row < rows) {
         const float4 *x4 = reinterpret_cast<const float4 *>(logits + row * cols);
 #pragma unroll
-        for (int k = 0; k < (PF ? NV : 1); ++k) vn[k] = __ldcs(x4 + (warp + k * kWarps) * 32 + lane);
+        for (int k = 0; k < (PF ? NV : 1); ++k)
+            if (FULL || warp + k * kWarps < nch) vn[k] = __ldcs(x4 + (warp + k * kWarps) * 32 + lane);
     }
     for (; row < rows; row += stride) {
         float4 v[NV];
@@ -701,23 +620,26 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
             if (row + stride < rows) {
                 const float4 *xn = reinterpret_cast<const float4 *>(logits + (row + stride) * cols);
 #pragma unroll
-                for (int k = 0; k < NV; ++k) vn[k] = __ldcs(xn + (warp + k * kWarps) * 32 + lane);
+                for (int k = 0; k < NV; ++k)
+                    if (FULL || warp + k * kWarps < nch) vn[k] = __ldcs(xn + (warp + k * kWarps) * 32 + lane);
             }
         } else {
             const float4 *x4 = reinterpret_cast<const float4 *>(logits + row * cols);
 #pragma unroll
-            for (int k = 0; k < NV; ++k) v[k] = __ldcs(x4 + (warp + k * kWarps) * 32 + lane);
+            for (int k = 0; k < NV; ++k)
+                if (FULL || warp + k * kWarps < nch) v[k] = __ldcs(x4 + (warp + k * kWarps) * 32 + lane);
         }
         // ---- block maxima -------------------------------------------------------------------------
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
+            if (!FULL && warp + k * kWarps >= nch) break;
             float mx = fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w));
             mx = lanes_max<LPB, REDUX>(mx);
             if ((lane % LPB) == 0) s_bmax[grp][(warp + k * kWarps) * BPW + lane / LPB] = mx;
         }
         gsync();
         // ---- scan over the blocks (the group's warp 0) ----------------------------------------------
-        if (warp == 0) scan_blocks<nb>(s_bmax[grp], s_mbefore[grp], &s_mfinal[grp], lambda, lane);
+        if (warp == 0) scan_blocks(nb, s_bmax[grp], s_mbefore[grp], &s_mfinal[grp], lambda, lane);
         gsync();
         const float mfinal = s_mfinal[grp];
         const int jmine = (warp + (lane / BPW) * kWarps) * BPW + lane % BPW;      // the block whose parameters I work out
@@ -726,31 +648,33 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
             // ---- codes, block exponents, the sum of the decoded weights ------------------------------
             uint32_t *c4 = reinterpret_cast<uint32_t *>(out.codes + row * cols);
             CodesBlockParams bp = {0.f, 0, 1, 0.f};
-            if (lane < NV * BPW) {
+            if (lane < NV * BPW && (FULL || jmine < nb)) {
                 bp = codes_block_params(s_mbefore[grp][jmine], s_bmax[grp][jmine], jmine == 0, lambda, mfinal);
                 out.block_exp[row * nb + jmine] = bp.bexp;
             }
             const int kindp = pack_kind<BPW>(bp.kind);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
+                if (!FULL && warp + k * kWarps >= nch) break;
                 const int src = k * BPW + lane / LPB;
                 const float mref = __shfl_sync(0xffffffffu, bp.mref, src);
                 const float be = __shfl_sync(0xffffffffu, bp.scale, src);
                 const int kp = __shfl_sync(0xffffffffu, kindp, src);
                 dsum += emit_codes(c4 + (warp + k * kWarps) * 32 + lane,
-                                   block_words<true>(v[k], mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
+                                   block_words(v[k], mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
             }
         } else {
             // ---- weights (already moved to the final max) and their sum ------------------------------
             BlockParams bp = {0.f, 0.f, 1};
-            if (lane < NV * BPW) bp = block_params(s_mbefore[grp][jmine], s_bmax[grp][jmine], jmine == 0, lambda, mfinal);
+            if (lane < NV * BPW && (FULL || jmine < nb)) bp = block_params(s_mbefore[grp][jmine], s_bmax[grp][jmine], jmine == 0, lambda, mfinal);
             const int kindp = pack_kind<BPW>(bp.kind);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
+                if (!FULL && warp + k * kWarps >= nch) break;
                 const int src = k * BPW + lane / LPB;
                 const float mref = __shfl_sync(0xffffffffu, bp.mref, src), scale = __shfl_sync(0xffffffffu, bp.scale, src);
                 const int kp = __shfl_sync(0xffffffffu, kindp, src);
-                v[k] = block_weights<true>(v[k], mref, scale, kp & 3, (kp & 4) != 0, reinterpret_cast<const float *>(s_rep),
+                v[k] = block_weights(v[k], mref, scale, kp & 3, (kp & 4) != 0, reinterpret_cast<const float *>(s_rep),
                                            reinterpret_cast<const float *>(s_lut), lane);
                 dsum += (v[k].x + v[k].y) + (v[k].z + v[k].w);
             }
@@ -775,8 +699,9 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
             float4 *p4 = reinterpret_cast<float4 *>(out.probs + row * cols);
 #pragma unroll
             for (int k = 0; k < NV; ++k)
-                __stcs(p4 + (warp + k * kWarps) * 32 + lane,
-                       make_float4(v[k].x * dinv, v[k].y * dinv, v[k].z * dinv, v[k].w * dinv));
+                if (FULL || warp + k * kWarps < nch)
+                    __stcs(p4 + (warp + k * kWarps) * 32 + lane,
+                           make_float4(v[k].x * dinv, v[k].y * dinv, v[k].z * dinv, v[k].w * dinv));
         }
         // (no barrier here: what the next row writes first, s_bmax, was last read before the third barrier
         // above; s_mfinal and s_red are written behind the next row's first and second barrier, which every
@@ -788,14 +713,15 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
 // Lane l holds the float4 number l of every 128-element chunk; a block of Algorithm 1 is a whole
 // chunk (BK = 128) or half of one (BK = 64).  Block maxima by a warp reduction, the scan replicated in
 // every lane (it is a handful of scalar steps per block), weights, warp-wide sum, write.  CODES: 8-bit output.
-template <int BK, int NV, bool CODES>
+template <int BK, int NV, bool CODES, bool FULL = true>
 __global__ void __launch_bounds__(512)
-softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda)
+softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda, int cols_)
 {
     __shared__ uint32_t s_lut[kLutN];
     __shared__ __align__(16) uint32_t s_rep[(16 + kLutNegN) * 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int LPB = BK / 4, BPW = 32 / LPB, cols = NV * 128, nb = cols / BK;
+    constexpr int LPB = BK / 4, BPW = 32 / LPB;
+    const int cols = FULL ? NV * 128 : cols_, nch = cols / 128, nb = cols / BK;
     static_assert(NV * BPW <= 32, "one block per lane");
     fill_tables<CODES, 512>(s_lut, s_rep, tid);
     __syncthreads();
@@ -806,9 +732,11 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
         float4 v[NV];
         float bmx[NV];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) v[k] = __ldcs(x4 + k * 32 + lane);
+        for (int k = 0; k < NV; ++k)
+            if (FULL || k < nch) v[k] = __ldcs(x4 + k * 32 + lane);
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
+            if (!FULL && k >= nch) break;
             float mx = fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w));
             mx = lanes_max<LPB>(mx);
             bmx[k] = mx;                                         // maximum of my block of chunk k
@@ -818,6 +746,7 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
         float m = -INFINITY, my_mb = -INFINITY, my_bm = -INFINITY;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
+            if (!FULL && k >= nch) break;
 #pragma unroll
             for (int q = 0; q < BPW; ++q) {
                 const float bj = __shfl_sync(0xffffffffu, bmx[k], q * LPB);
@@ -831,18 +760,19 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
         if constexpr (CODES) {
             uint32_t *c4 = reinterpret_cast<uint32_t *>(out.codes + row * cols);
             CodesBlockParams bp = {0.f, 0, 1, 0.f};
-            if (lane < NV * BPW) {
+            if (lane < (FULL ? NV * BPW : nb)) {
                 bp = codes_block_params(my_mb, my_bm, lane == 0, lambda, mfinal);
                 out.block_exp[row * nb + lane] = bp.bexp;
             }
             const int kindp = pack_kind<BPW>(bp.kind);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
+                if (!FULL && k >= nch) break;
                 const int src = k * BPW + myq;
                 const float mref = __shfl_sync(0xffffffffu, bp.mref, src);
                 const float be = __shfl_sync(0xffffffffu, bp.scale, src);
                 const int kp = __shfl_sync(0xffffffffu, kindp, src);
-                dsum += emit_codes(c4 + k * 32 + lane, block_words<true>(v[k], mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
+                dsum += emit_codes(c4 + k * 32 + lane, block_words(v[k], mref, (kp & 4) != 0, s_rep, s_lut, lane), be);
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
@@ -850,14 +780,15 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
         } else {
             float4 *p4 = reinterpret_cast<float4 *>(out.probs + row * cols);
             BlockParams bp = {0.f, 0.f, 1};
-            if (lane < NV * BPW) bp = block_params(my_mb, my_bm, lane == 0, lambda, mfinal);
+            if (lane < (FULL ? NV * BPW : nb)) bp = block_params(my_mb, my_bm, lane == 0, lambda, mfinal);
             const int kindp = pack_kind<BPW>(bp.kind);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
+                if (!FULL && k >= nch) break;
                 const int src = k * BPW + myq;
                 const float mref = __shfl_sync(0xffffffffu, bp.mref, src), scale = __shfl_sync(0xffffffffu, bp.scale, src);
                 const int kp = __shfl_sync(0xffffffffu, kindp, src);
-                v[k] = block_weights<true>(v[k], mref, scale, kp & 3, (kp & 4) != 0, reinterpret_cast<const float *>(s_rep),
+                v[k] = block_weights(v[k], mref, scale, kp & 3, (kp & 4) != 0, reinterpret_cast<const float *>(s_rep),
                                            reinterpret_cast<const float *>(s_lut), lane);
                 dsum += (v[k].x + v[k].y) + (v[k].z + v[k].w);
             }
@@ -866,7 +797,8 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
             const float dinv = 1.f / dsum;
 #pragma unroll
             for (int k = 0; k < NV; ++k)
-                __stcs(p4 + k * 32 + lane, make_float4(v[k].x * dinv, v[k].y * dinv, v[k].z * dinv, v[k].w * dinv));
+                if (FULL || k < nch)
+                    __stcs(p4 + k * 32 + lane, make_float4(v[k].x * dinv, v[k].y * dinv, v[k].z * dinv, v[k].w * dinv));
         }
     }
 }
@@ -881,90 +813,6 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
 // bits, so the low byte of its fp32 pattern is free for the code.  Blocks whose T are all <= 0 take their
 // table word from a bank-replicated copy keyed by the top bits of -T * 2^-120 (as in the float-output
 // kernels above).
-// Any row length that is a multiple of 128: one CTA per row at a time; pass 1 block maxima (the HBM
-// read), scan by warp 0, pass 2 re-reads the row (from L2), looks every T up and sums the decoded weights.
-template <int BK, int THREADS, bool FAST>
-__global__ void __launch_bounds__(THREADS)
-softmax_rows_codes_generic_kernel(const float *__restrict__ logits, uint8_t *__restrict__ codes,
-                                  int32_t *__restrict__ block_exp, float *__restrict__ row_d, int64_t rows, int cols,
-                                  int lambda)
-{
-    __shared__ float s_bmax[kSrMaxBlocks];
-    __shared__ float s_mbefore[kSrMaxBlocks];
-    __shared__ uint32_t s_lut[kLutN];
-    __shared__ __align__(16) uint32_t s_rep[FAST ? (16 + kLutNegN) * 32 : 32];
-    __shared__ float s_red[THREADS / 32];
-    __shared__ float s_mfinal;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int kWarps = THREADS / 32;
-    constexpr int LPB = BK / 4, BPW = 32 / LPB;
-    const int nb = cols / BK, nchunks = cols / 128;
-    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = w0_word(g_w0.v[i]);
-    for (int e = tid; FAST && e < 16 + kLutNegN; e += THREADS) {
-        const uint32_t u = w0_word((e < 16) ? 1.f : g_w0.v[e - 16]);
-        const uint4 u4 = make_uint4(u, u, u, u);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) reinterpret_cast<uint4 *>(s_rep)[e * 8 + i] = u4;
-    }
-    __syncthreads();
-    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-        const float4 *x4 = reinterpret_cast<const float4 *>(logits + row * cols);
-        uint32_t *c4 = reinterpret_cast<uint32_t *>(codes + row * cols);
-        for (int ch = warp; ch < nchunks; ch += kWarps) {
-            const float4 x = __ldg(x4 + ch * 32 + lane);
-            float mx = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
-            mx = lanes_max<LPB>(mx);
-            if ((lane % LPB) == 0) s_bmax[ch * BPW + lane / LPB] = mx;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            bool rs; float dl;
-            float m = row_block_update(-INFINITY, s_bmax[0], true, lambda, &rs, &dl);
-            if (lane == 0) s_mbefore[0] = -INFINITY;
-            for (int base = 1; base < nb; base += 32) {
-                const int j = base + lane;
-                const bool valid = j < nb;
-                const float mj = valid ? s_bmax[j] : -INFINITY;
-                bool pending = valid;
-                while (true) {
-                    const bool pred = pending && fmaf(mj, kLog2e, -m) >= 1.1920928955078125e-07f;
-                    const unsigned b = __ballot_sync(0xffffffffu, pred);
-                    if (b == 0u) { if (pending) s_mbefore[j] = m; break; }
-                    const int l = __ffs(b) - 1;
-                    if (pending && lane <= l) { s_mbefore[j] = m; pending = false; }
-                    const float ml = __shfl_sync(0xffffffffu, mj, l);
-                    m = row_block_update(m, ml, false, lambda, &rs, &dl);
-                }
-            }
-            if (lane == 0) s_mfinal = m;
-        }
-        __syncthreads();
-        const float mfinal = s_mfinal;
-        float dsum = 0.f;
-        for (int ch = warp; ch < nchunks; ch += kWarps) {
-            const float4 x = __ldg(x4 + ch * 32 + lane);
-            const int j = ch * BPW + lane / LPB;
-            const CodesBlockParams bp = codes_block_params(s_mbefore[j], s_bmax[j], j == 0, lambda, mfinal);
-            // some lane of the warp holds a block with a positive T: voted by the whole warp
-            const bool any_pos = __any_sync(0xffffffffu, bp.kind == 2);
-            const uint4 e = block_words<FAST>(x, bp.mref, any_pos, s_rep, s_lut, lane);
-            dsum += ((__uint_as_float(e.x & 0xFFFFFF00u) + __uint_as_float(e.y & 0xFFFFFF00u)) +
-                     (__uint_as_float(e.z & 0xFFFFFF00u) + __uint_as_float(e.w & 0xFFFFFF00u))) * bp.scale;
-            __stcs(c4 + ch * 32 + lane, (e.x & 0xFFu) | ((e.y & 0xFFu) << 8) | ((e.z & 0xFFu) << 16) | (e.w << 24));
-            if ((lane % LPB) == 0) block_exp[row * nb + j] = bp.bexp;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-        if (lane == 0) s_red[warp] = dsum;
-        __syncthreads();
-        if (tid == 0) {
-            float t = 0.f;
-            for (int i = 0; i < kWarps; ++i) t += s_red[i];
-            row_d[row] = t;
-        }
-        __syncthreads();   // s_bmax / s_mbefore / s_red are reused by the next row
-    }
-}
 
 template <int BK>
 inline baps_status softmax_rows_codes_dispatch(const float *logits, uint8_t *codes, int32_t *block_exp, float *row_d,
@@ -979,33 +827,41 @@ inline baps_status softmax_rows_codes_dispatch(const float *logits, uint8_t *cod
     auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
             return BAPS_ERR_CUDA;
-        kernel<<<grid_for(ctas_per_sm), threads, dyn, st>>>(logits, out, rows, lambda);
+        kernel<<<grid_for(ctas_per_sm), threads, dyn, st>>>(logits, out, rows, lambda, cols);
         return BAPS_OK;
     };
     auto group = [&](auto kernel, int threads, int groups, int ctas) {
         const int64_t want = (rows + groups - 1) / groups, cap = (int64_t)num_sms * ctas;
-        kernel<<<(int)(want < cap ? want : cap), threads * groups, 0, st>>>(logits, out, rows, lambda);
+        kernel<<<(int)(want < cap ? want : cap), threads * groups, 0, st>>>(logits, out, rows, lambda, cols);
+        return BAPS_OK;
     };
-    switch (cols) {
-    case 1024: {
+    auto warp_rows = [&](auto kernel) {
         const int64_t want = (rows + 15) / 16, cap = (int64_t)num_sms * 32;
-        softmax_rows_warp_kernel<BK, 8, true><<<(int)(want < cap ? want : cap), 512, 0, st>>>(logits, out, rows, lambda);
-        break;
-    }
-    case 2048:  group(softmax_rows_group_kernel<BK, 128, 4, 4, true, true>, 128, 4, 16); break;
-    case 4096:  group(softmax_rows_group_kernel<BK, 256, 4, 4, true, true>, 256, 4, 4); break;
-    case 8192:  group(softmax_rows_group_kernel<BK, 256, 8, 4, true, false>, 256, 4, 4); break;
-    case 16384: if (ring(softmax_rows_ring_kernel<BK, 512, true>, 512, 65536, 2) != BAPS_OK) return BAPS_ERR_CUDA; break;
-    case 32768: if (ring(softmax_rows_ring_kernel<BK, 1024, true>, 1024, 131072, 2) != BAPS_OK) return BAPS_ERR_CUDA; break;
-    case 65536: if (ring(softmax_rows_quarters_kernel<BK, true>, 1024, 196608, 2) != BAPS_OK) return BAPS_ERR_CUDA; break;
+        kernel<<<(int)(want < cap ? want : cap), 512, 0, st>>>(logits, out, rows, lambda, cols);
+        return BAPS_OK;
+    };
+    baps_status rc;
+    switch (cols) {
+    case 1024:  rc = warp_rows(softmax_rows_warp_kernel<BK, 8, true>); break;
+    case 2048:  rc = group(softmax_rows_group_kernel<BK, 128, 4, 4, true, true>, 128, 4, 16); break;
+    case 4096:  rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, true, true, true>, 256, 4, 4); break;
+    case 8192:  rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, true, false>, 256, 4, 4); break;
+    case 16384: rc = ring(softmax_rows_ring_kernel<BK, 512, true, true>, 512, 65536, 2); break;
+    case 32768: rc = ring(softmax_rows_ring_kernel<BK, 1024, true>, 1024, 131072, 2); break;
+    case 65536: rc = ring(softmax_rows_quarters_kernel<BK, true>, 1024, 196608, 2); break;
     default:
-        // other lengths re-read the row: large CTAs for long rows so that the re-read finds it in L2
-        if (cols > 8192)
-            softmax_rows_codes_generic_kernel<BK, 1024, true><<<grid_for(2), 1024, 0, st>>>(logits, codes, block_exp, row_d, rows, cols, lambda);
-        else
-            softmax_rows_codes_generic_kernel<BK, 256, false><<<grid_for(8), 256, 0, st>>>(logits, codes, block_exp, row_d, rows, cols, lambda);
+        // Any other length by the next larger of these shapes, with the vectors past the end left out
+        // (chunks of 128 columns are dealt to warps, so every test for the end is the same for a whole warp).
+        if (cols < 1024) rc = warp_rows(softmax_rows_warp_kernel<BK, 8, true, false>);
+        else if (cols < 2048) rc = group(softmax_rows_group_kernel<BK, 128, 4, 4, true, true, true, false>, 128, 4, 16);
+        else if (cols < 4096) rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, true, true, true, false>, 256, 4, 4);
+        else if (cols < 8192) rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, true, false, true, false>, 256, 4, 4);
+        else if (cols < 16384) rc = ring(softmax_rows_ring_kernel<BK, 512, true, true, false>, 512, cols * 4, 2);
+        else if (cols < 32768) rc = ring(softmax_rows_ring_kernel<BK, 1024, true, true, false>, 1024, cols * 4, 2);
+        else rc = ring(softmax_rows_quarters_kernel<BK, true, false>, 1024, 196608, 2);
         break;
     }
+    if (rc != BAPS_OK) return rc;
     return launch_status();
 }
 
@@ -1022,7 +878,7 @@ inline baps_status softmax_rows_dispatch(const float *logits, float *probs, int6
     auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
             return BAPS_ERR_CUDA;
-        kernel<<<grid_for(ctas_per_sm), threads, dyn, st>>>(logits, out, rows, lambda);
+        kernel<<<grid_for(ctas_per_sm), threads, dyn, st>>>(logits, out, rows, lambda, cols);
         return BAPS_OK;
     };
     // Grids: several times the CTAs that are resident at once (a few rows per CTA), so that the hardware
@@ -1034,29 +890,36 @@ inline baps_status softmax_rows_dispatch(const float *logits, float *probs, int6
     // the current row's passes.
     auto group = [&](auto kernel, int threads, int groups, int ctas) {
         const int64_t want = (rows + groups - 1) / groups, cap = (int64_t)num_sms * ctas;
-        kernel<<<(int)(want < cap ? want : cap), threads * groups, 0, st>>>(logits, out, rows, lambda);
+        kernel<<<(int)(want < cap ? want : cap), threads * groups, 0, st>>>(logits, out, rows, lambda, cols);
+        return BAPS_OK;
     };
-    switch (cols) {
-    case 1024: {
+    auto warp_rows = [&](auto kernel) {
         const int64_t want = (rows + 15) / 16, cap = (int64_t)num_sms * 32;
-        softmax_rows_warp_kernel<BK, 8, false><<<(int)(want < cap ? want : cap), 512, 0, st>>>(logits, out, rows, lambda);
-        break;
-    }
-    case 2048: group(softmax_rows_group_kernel<BK, 128, 4, 4, false, true>, 128, 4, 16); break;
-    case 4096: group(softmax_rows_group_kernel<BK, 256, 4, 4, false, true, false>, 256, 4, 4); break;
-    case 8192: group(softmax_rows_group_kernel<BK, 256, 8, 4, false, false>, 256, 4, 4); break;
-    case 16384: if (ring(softmax_rows_ring_kernel<BK, 512, false, false>, 512, 65536, 2) != BAPS_OK) return BAPS_ERR_CUDA; break;
-    case 32768: if (ring(softmax_rows_ring_kernel<BK, 1024, false>, 1024, 131072, 2) != BAPS_OK) return BAPS_ERR_CUDA; break;
-    case 65536: if (ring(softmax_rows_quarters_kernel<BK, false>, 1024, 196608, 2) != BAPS_OK) return BAPS_ERR_CUDA; break;
+        kernel<<<(int)(want < cap ? want : cap), 512, 0, st>>>(logits, out, rows, lambda, cols);
+        return BAPS_OK;
+    };
+    baps_status rc;
+    switch (cols) {
+    case 1024:  rc = warp_rows(softmax_rows_warp_kernel<BK, 8, false>); break;
+    case 2048:  rc = group(softmax_rows_group_kernel<BK, 128, 4, 4, false, true>, 128, 4, 16); break;
+    case 4096:  rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, false, true, false>, 256, 4, 4); break;
+    case 8192:  rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, false, false>, 256, 4, 4); break;
+    case 16384: rc = ring(softmax_rows_ring_kernel<BK, 512, false, false>, 512, 65536, 2); break;
+    case 32768: rc = ring(softmax_rows_ring_kernel<BK, 1024, false>, 1024, 131072, 2); break;
+    case 65536: rc = ring(softmax_rows_quarters_kernel<BK, false>, 1024, 196608, 2); break;
     default:
-        if (cols >= 32768) {
-            // long rows are re-read in passes 2 and 3: few enough CTAs that the rows in flight stay in L2
-            softmax_rows_generic_kernel<BK, 1024, true><<<grid_for(2), 1024, 0, st>>>(logits, probs, rows, cols, lambda);
-        } else {
-            softmax_rows_generic_kernel<BK, 256, false><<<grid_for(8), 256, 0, st>>>(logits, probs, rows, cols, lambda);
-        }
+        // Any other length by the next larger of these shapes, with the vectors past the end left out
+        // (chunks of 128 columns are dealt to warps, so every test for the end is the same for a whole warp).
+        if (cols < 1024) rc = warp_rows(softmax_rows_warp_kernel<BK, 8, false, false>);
+        else if (cols < 2048) rc = group(softmax_rows_group_kernel<BK, 128, 4, 4, false, true, true, false>, 128, 4, 16);
+        else if (cols < 4096) rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, false, true, false, false>, 256, 4, 4);
+        else if (cols < 8192) rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, false, false, true, false>, 256, 4, 4);
+        else if (cols < 16384) rc = ring(softmax_rows_ring_kernel<BK, 512, false, false, false>, 512, cols * 4, 2);
+        else if (cols < 32768) rc = ring(softmax_rows_ring_kernel<BK, 1024, false, true, false>, 1024, cols * 4, 2);
+        else rc = ring(softmax_rows_quarters_kernel<BK, false, false>, 1024, 196608, 2);
         break;
     }
+    if (rc != BAPS_OK) return rc;
     return launch_status();
 }
 

@@ -167,3 +167,16 @@ def test_softmax_rows_with_masked_entries(cols):
     assert (got[:, 256:384] == 0).all()
     gate_softmax_rows(got, probs, margin, allow, what=f"masked cols={cols}")
     _check_codes(x, 128, f"masked codes cols={cols}")
+
+
+@pytest.mark.parametrize("block_k", [64, 128])
+@pytest.mark.parametrize("chunks", [1, 7, 9, 15, 17, 31, 33, 63, 65, 127, 129, 255, 257, 383, 384, 385, 511])
+def test_softmax_rows_any_length(chunks, block_k):
+    """Row lengths on both sides of every change of kernel (chunks of 128 columns), both outputs."""
+    cols = 128 * chunks
+    x = workloads.make_rows(5 if chunks < 128 else 2, cols, var=4.0, seed=chunks + block_k)
+    x += torch.linspace(-3, 3, cols)[None, :]                       # some blocks raise the max
+    got = binding.baps_softmax_rows(x.cuda(), block_k=block_k).cpu().numpy()
+    probs, margin, allow = oracle.softmax_rows(x.numpy(), block_k=block_k, want_allow=True)
+    gate_softmax_rows(got, probs, margin, allow, what=f"chunks={chunks} bk={block_k}")
+    _check_codes(x, block_k, f"chunks={chunks} bk={block_k}")
