@@ -1,7 +1,7 @@
 // Fused BAPS attention forward on the 5th-generation tensor cores (tcgen05, sm_100a).
 //
-// One CTA owns two consecutive 128-row query tiles (t = 0, 1) of one (batch, head) and walks the
-// key tiles j in increasing order (Algorithm 1: tile 0 is the high-precision set B0, all later
+// One CTA owns two consecutive 128-row query tiles (t = 0, 1; small grids: one, see one_tile_per_cta) of one
+// (batch, head) and walks the key tiles j in increasing order (Algorithm 1: tile 0 is the high-precision set B0, all later
 // tiles are 8-bit tiles).  The unit of work is a task (t, j): S = Q_t K_j^T, softmax bookkeeping
 // and weights P, O_t += P V_j.  Tasks run in the order (0,0) (1,0) (0,1) (1,1) ...; task k uses
 // score buffer k % 2 of tensor memory, so the tensor core forms the scores of task k + 1 while
@@ -244,7 +244,8 @@ __device__ __forceinline__ float max8(const uint32_t *x)
 // kB0Last: B0 = {first, last visible key tile} (compile-time, so that the usual order pays nothing).
 // kMode (BAPS_MODE_*): Algorithm 1, the exact mode, or -- kExp2 below -- the "Exp2 HiF8" setup of Section 4.1 (Eq. (2) with a real-valued max, weights and
 // rescale factor through the 8-bit exponent table); otherwise Algorithm 1 or the exact mode.
-template <int D, int kMode, bool kQK8 = false, bool kB0Last = false>
+// kOne: a CTA owns one query tile instead of two (small grids, see one_tile_per_cta; always with kB0Last).
+template <int D, int kMode, bool kQK8 = false, bool kB0Last = false, bool kOne = kB0Last>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                     const __grid_constant__ CUtensorMap mv, const AttnTcParams p)
@@ -276,12 +277,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     // With B0 = {first, last} the key tiles are visited in the order 0, last, 1, ..., last - 1, and
     // "last" differs between neighbouring query tiles of a causal problem, so the two query tiles of
     // a pair could not share their K / V stream: the CTA then owns a single query tile (t = 0).
-    const int qbase = kB0Last ? pair : 2 * pair;        // first query tile of this CTA
+    const int qbase = kOne ? pair : 2 * pair;        // first query tile of this CTA
     int jm[2];                                   // number of key tiles of each query tile
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
         const int qi = qbase + t;
-        jm[t] = (qi < p.nq && !(kB0Last && t == 1)) ? (p.causal ? qi + 1 : nk) : 0;
+        jm[t] = (qi < p.nq && !(kOne && t == 1)) ? (p.causal ? qi + 1 : nk) : 0;
     }
     const int J = jm[0] > jm[1] ? jm[0] : jm[1];
     const int nb0 = (kB0Last && J >= 2) ? 2 : 1;        // number of high-precision (B0) steps
@@ -291,11 +292,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     const int kv_row0 = (b * p.Hkv + hk) * p.S;
 
     // ---- setup --------------------------------------------------------------------------------
-    // kEarly (D = 64, where a CTA lives for few tasks): the producer lane initialises the barriers itself and
+    // kEarly (D = 64 or one query tile, where a CTA lives for few tasks): the producer lane initialises the barriers itself and
     // starts the Q tiles and the first ring-full of K / V tiles before the CTA-wide barrier, so that the copies
-    // are on their way while the rest of the CTA is still setting up.  (At D = 128 the same change made the
-    // steady state 2 % slower, so that path keeps the plain order.)
-    constexpr bool kEarly = (D == 64);
+    // are on their way while the rest of the CTA is still setting up.  (With two tiles at D = 128 the same
+    // change made the steady state 2 % slower, so that path keeps the plain order.)
+    constexpr bool kEarly = (D == 64) || kOne;
     constexpr int kQkBoxes = kQK8 ? 1 : D / 64;
     constexpr uint32_t kQkTileBytes = kQK8 ? 128 * D : L::kTileBytes;
     const int n_early = kEarly ? (2 * J < L::kStages ? 2 * J : L::kStages) : 0;   // loads that need no free stage
@@ -728,8 +729,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
 
         if (J > 0) load_scores(0);
         for (int j = 0; j < J; ++j) {
-            if (j < jm[0]) task(std::integral_constant<int, 0>{}, j, j < jm[1] || j + 1 < J);
-            if (j < jm[1]) task(std::integral_constant<int, 1>{}, j, j + 1 < J);
+            if (j < jm[0]) task(std::integral_constant<int, 0>{}, j, (!kOne && j < jm[1]) || j + 1 < J);
+            if constexpr (!kOne)
+                if (j < jm[1]) task(std::integral_constant<int, 1>{}, j, j + 1 < J);
         }
         const bool ok = (*s_abort == 0);
 
@@ -807,7 +809,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
                 p.restarts[(size_t)(b * p.H + h) * p.nq + qi] = n_restart[T];
         };
         finish(std::integral_constant<int, 0>{});
-        finish(std::integral_constant<int, 1>{});
+        if constexpr (!kOne) finish(std::integral_constant<int, 1>{});
     }
 
     // ---- teardown ---------------------------------------------------------------------------------
@@ -816,10 +818,36 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     if (warp == 16) { __syncwarp(); tmem_dealloc(tmem, 512); }
 }
 
+// One query tile per CTA or two?  Two share the K / V stream and the set-up of the CTA, and a task (one score
+// tile, 1.35 us) waits less on the one before it; one halves the chain of tasks that the longest CTA walks
+// through, which is what a grid that does not fill the SMs several times over takes.  Estimate of both in units
+// of a two-tile task, SMs filled longest CTA first: the longest CTA or the average load of an SM, whichever is
+// larger (all CTAs of a bidirectional problem are equally long: whole waves).  Besides its tasks a CTA costs
+// kFixedTwo / kFixedOne (set-up, first scores, epilogues).  Measured, two tiles -> one (D = 128, causal, heads x
+// tokens): 4 x 512 15.8 -> 11.4 us, 8 x 4096 90.8 -> 58.1, 32 x 1024 28.8 -> 23.7, 1 x 16384 326 -> 215; and
+// where two stay: 16 x 4096 90.6 -> 111, 32 x 2048 53.7 -> 67, 4 x 32768 1190 -> 1501.
+static inline bool one_tile_per_cta(long long heads, int nq, bool causal, int num_sms)
+{
+    constexpr double kFixedTwo = 4.5, kFixedOne = 3.5, kTaskOne = 1.25;
+    const long long ctas2 = heads * ((nq + 1) / 2), ctas1 = heads * nq;
+    const double longest1 = kTaskOne * nq + kFixedOne, longest2 = (causal || nq == 1 ? 2 * nq - 1 : 2 * nq) + kFixedTwo;
+    double t1, t2;
+    if (causal) {
+        const double tasks = (double)heads * nq * (nq + 1) / 2;
+        const double load1 = (kTaskOne * tasks + kFixedOne * ctas1) / num_sms, load2 = (tasks + kFixedTwo * ctas2) / num_sms;
+        t1 = load1 > longest1 ? load1 : longest1;
+        t2 = load2 > longest2 ? load2 : longest2;
+    } else {
+        t1 = (double)((ctas1 + num_sms - 1) / num_sms) * longest1;
+        t2 = (double)((ctas2 + num_sms - 1) / num_sms) * longest2;
+    }
+    return t1 < t2;
+}
+
 // Host side: tensor maps, one-time table initialisation, launch.
 static inline baps_status attention_tc_launch(const void *q, const void *k, const void *v, void *out, int B, int H,
                                        int Hkv, int S, int D, int causal, int lambda, int mode, int b0_last, float c,
-                                       const baps_stats &st, int /*num_sms*/, cudaStream_t stream,
+                                       const baps_stats &st, int num_sms, cudaStream_t stream,
                                        const float *q_scale = nullptr, const float *k_scale = nullptr)
 {
     const bool qk8 = q_scale != nullptr;               // Q, K are E4M3 codes with per-tile scales
@@ -839,7 +867,9 @@ static inline baps_status attention_tc_launch(const void *q, const void *k, cons
     p.B = B; p.H = H; p.Hkv = Hkv; p.S = S; p.causal = causal; p.lambda = lambda; p.mode = mode; p.c = c;
     p.b0_last = (b0_last && mode == BAPS_MODE_E2E_HIF8) ? 1 : 0;
     p.q_scale = q_scale; p.k_scale = k_scale;
-    p.nq = S / 128; p.npairs = p.b0_last ? p.nq : (p.nq + 1) / 2;
+    p.nq = S / 128;
+    const bool one = p.b0_last || (mode == BAPS_MODE_E2E_HIF8 && one_tile_per_cta((long long)B * H, p.nq, causal != 0, num_sms));
+    p.npairs = one ? p.nq : (p.nq + 1) / 2;
     const long long nblocks = (long long)p.npairs * B * H;
     if (nblocks > 0x7fffffffLL) return BAPS_ERR_UNSUPPORTED;
     auto launch = [&](auto kernel, int sm) -> baps_status {
@@ -855,18 +885,21 @@ static inline baps_status attention_tc_launch(const void *q, const void *k, cons
         if (mode == kExp2m) return launch(attention_tc_kernel<128, kExp2m, true, false>, TcLayout<128>::kDynBytes);
         if (mode == kExact) return launch(attention_tc_kernel<128, kExact, true, false>, TcLayout<128>::kDynBytes);
         return b0l ? launch(attention_tc_kernel<128, kE2E, true, true>, TcLayout<128>::kDynBytes)
-                   : launch(attention_tc_kernel<128, kE2E, true, false>, TcLayout<128>::kDynBytes);
+                   : one ? launch(attention_tc_kernel<128, kE2E, true, false, true>, TcLayout<128>::kDynBytes)
+                         : launch(attention_tc_kernel<128, kE2E, true, false, false>, TcLayout<128>::kDynBytes);
     }
     if (D == 128) {
         if (mode == kExp2m) return launch(attention_tc_kernel<128, kExp2m, false, false>, TcLayout<128>::kDynBytes);
         if (mode == kExact) return launch(attention_tc_kernel<128, kExact, false, false>, TcLayout<128>::kDynBytes);
         return b0l ? launch(attention_tc_kernel<128, kE2E, false, true>, TcLayout<128>::kDynBytes)
-                   : launch(attention_tc_kernel<128, kE2E, false, false>, TcLayout<128>::kDynBytes);
+                   : one ? launch(attention_tc_kernel<128, kE2E, false, false, true>, TcLayout<128>::kDynBytes)
+                         : launch(attention_tc_kernel<128, kE2E, false, false, false>, TcLayout<128>::kDynBytes);
     }
     if (mode == kExp2m) return launch(attention_tc_kernel<64, kExp2m, false, false>, TcLayout<64>::kDynBytes);
     if (mode == kExact) return launch(attention_tc_kernel<64, kExact, false, false>, TcLayout<64>::kDynBytes);
     return b0l ? launch(attention_tc_kernel<64, kE2E, false, true>, TcLayout<64>::kDynBytes)
-               : launch(attention_tc_kernel<64, kE2E, false, false>, TcLayout<64>::kDynBytes);
+               : one ? launch(attention_tc_kernel<64, kE2E, false, false, true>, TcLayout<64>::kDynBytes)
+                     : launch(attention_tc_kernel<64, kE2E, false, false, false>, TcLayout<64>::kDynBytes);
 }
 
 } // namespace baps

@@ -243,3 +243,19 @@ def test_restart_rates_rejects_small_scratch():
     with pytest.raises(binding.BapsError):
         binding.baps_attention_restart_rates(q, k, v, causal=True,
                                              scratch=torch.empty(3, dtype=torch.int32, device="cuda"))
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("S", [128, 384, 512])
+def test_one_and_two_query_tiles_per_cta_agree(S, D, causal):
+    """A few heads (one query tile per CTA) and the same heads repeated until the SMs are full several times
+    over (two tiles per CTA, an odd one left over at S = 384) give the same bits."""
+    g = torch.Generator(device="cuda"); g.manual_seed(S + D)
+    q, k, v = (torch.randn(1, h, S, D, device="cuda", generator=g).bfloat16() for h in (6, 2, 2))
+    few = binding.baps_attention_fwd_ex(q, k, v, causal=causal, block_q=128, block_k=128)
+    n = 256
+    many = binding.baps_attention_fwd_ex(*(t.repeat(n, 1, 1, 1) for t in (q, k, v)), causal=causal, block_q=128, block_k=128)
+    for a, b in ((few.out, many.out), (few.out_f32, many.out_f32), (few.row_m, many.row_m), (few.row_d, many.row_d),
+                 (few.restarts, many.restarts)):
+        assert torch.equal(a.expand_as(b), b)
