@@ -88,6 +88,7 @@ attention_f32_kernel(const AttnF32Params p)
     __shared__ float s_alpha[R], s_dinv[R];
     __shared__ int s_flag[3];
 
+    allow_next_kernel();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x % kAfCluster, tile = blockIdx.x / kAfCluster, h = blockIdx.y, b = blockIdx.z;
     const int D = p.D, S = p.S;
@@ -117,6 +118,9 @@ attention_f32_kernel(const AttnF32Params p)
         }
         cp_async_commit();
     };
+    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = g_w0.v[i];
+    if (tid < 3) s_flag[tid] = 0;
+    qh = await_previous_kernel(qh);
     fetch(s_K, lay.ks, kh);
     for (int i = tid; i < R * lay.Dp; i += THREADS) {
         const int r = i / lay.Dp, d = i % lay.Dp;
@@ -125,8 +129,6 @@ attention_f32_kernel(const AttnF32Params p)
     if (lay.Dp > D)                                          // the copies never touch the padding
         for (int i = tid; i < BLK * (lay.Dp - D); i += THREADS)
             s_K[(i / (lay.Dp - D)) * lay.ks + D + i % (lay.Dp - D)] = 0.f;
-    for (int i = tid; i < kLutN; i += THREADS) s_lut[i] = g_w0.v[i];
-    if (tid < 3) s_flag[tid] = 0;
     // every CTA of the cluster has cleared its flags before another one may set them
     asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");

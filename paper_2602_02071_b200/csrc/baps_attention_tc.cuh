@@ -85,6 +85,13 @@ __device__ __forceinline__ float lds_f32(uint32_t addr)
     asm("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
     return v;
 }
+// global load that stays behind the wait for the kernel ahead (await_previous_kernel), as volatile statements do
+__device__ __forceinline__ float ldg_f32(const float *p)
+{
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
@@ -263,6 +270,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::kMiscOff);
     volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L::kMiscOff + 4);
 
+    allow_next_kernel();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // ---- work assignment: heavy (late) query tiles first; the g query heads of one kv head adjacent
@@ -291,6 +299,20 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     const int q_row0 = (b * p.H + h) * p.S + qbase * 128;           // row in the [B*H*S, D] view
     const int kv_row0 = (b * p.Hkv + hk) * p.S;
 
+    // Tables of the softmax warps, built while the first Q / K tiles are on their way: the 32-way replicated
+    // fast-path table (one global load per entry, copies written with 16-byte stores) and the plain full table.
+    auto fill_tables = [&] {
+        float4 *rep = reinterpret_cast<float4 *>(smem + L::kLutRepOff);
+        for (int e = tid; e < kLutRepEntries; e += kTcSoftmaxWarps * 32) {
+            const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
+            const float4 w4 = make_float4(w, w, w, w);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) rep[e * 8 + i] = w4;
+        }
+        float *full = reinterpret_cast<float *>(smem + L::kLutFullOff);
+        for (int i = tid; i < kLutN; i += kTcSoftmaxWarps * 32) full[i] = g_w0.v[i];
+    };
+
     // ---- setup --------------------------------------------------------------------------------
     // kEarly (D = 64 or one query tile, where a CTA lives for few tasks): the producer lane initialises the barriers itself and
     // starts the Q tiles and the first ring-full of K / V tiles before the CTA-wide barrier, so that the copies
@@ -312,6 +334,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
                 }
                 for (int s = 0; s < L::kStages; ++s) { mbar_init(bar(BKF + s), 1); mbar_init(bar(BKE + s), 1); }
                 mbar_fence_init();
+                await_previous_kernel();
                 const int nvalid = (jm[0] > 0) + (jm[1] > 0);
                 mbar_arrive_expect_tx(bar(BQ), (uint32_t)nvalid * kQkTileBytes);
                 for (int t = 0; t < 2; ++t)
@@ -332,8 +355,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
                 }
             }
             __syncwarp();
-            tmem_alloc(smem_u32(s_tmem), 512); tmem_relinquish();
         }
+        if (warp == 17) { tmem_alloc(smem_u32(s_tmem), 512); tmem_relinquish(); }
+        if (warp < kTcSoftmaxWarps) fill_tables();
     } else {
         if (tid == 0) {
             mbar_init(bar(BQ), 1);
@@ -364,6 +388,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
         // ======================= TMA producer ==================================================
         if (lane == 0) {
             if constexpr (!kEarly) {
+                await_previous_kernel();
                 const int nvalid = (jm[0] > 0) + (jm[1] > 0);
                 mbar_arrive_expect_tx(bar(BQ), (uint32_t)nvalid * kQkTileBytes);
                 for (int t = 0; t < 2; ++t)
@@ -510,21 +535,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
         // ======================= softmax warps ==================================================
-        // Tables, built while the first Q / K tiles are on their way: the 32-way replicated fast-path
-        // table (one global load per entry, copies written with 16-byte stores) and the plain full
-        // table.  Only the softmax warps read them, so a barrier among these warps suffices.
-        {
-            float4 *rep = reinterpret_cast<float4 *>(smem + L::kLutRepOff);
-            for (int e = tid; e < kLutRepEntries; e += kTcSoftmaxWarps * 32) {
-                const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
-                const float4 w4 = make_float4(w, w, w, w);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) rep[e * 8 + i] = w4;
-            }
-            float *full = reinterpret_cast<float *>(smem + L::kLutFullOff);
-            for (int i = tid; i < kLutN; i += kTcSoftmaxWarps * 32) full[i] = g_w0.v[i];
+        // (kEarly: the tables were filled before the CTA-wide barrier, while a kernel ahead was still draining)
+        if constexpr (!kEarly) {
+            fill_tables();
             named_bar_sync(6, kTcSoftmaxWarps * 32);
         }
+        await_previous_kernel();
         const int q4 = warp & 3;                 // TMEM lane quarter: rows 32 q4 .. 32 q4 + 31
         const int cq = warp >> 2;                // key column quarter: columns 32 cq .. 32 cq + 31
         const int row = q4 * 32 + lane;
@@ -567,8 +583,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
             // and of the key tile when Q and K are 8-bit (powers of two: the product is exact)
             float c = c_base;
             if constexpr (kQK8)
-                c = c_base * __ldg(p.q_scale + (size_t)(b * p.H + h) * p.nq + qi) *
-                    __ldg(p.k_scale + (size_t)(b * p.Hkv + hk) * nk + key_tile(j));
+                c = c_base * ldg_f32(p.q_scale + (size_t)(b * p.H + h) * p.nq + qi) *
+                    ldg_f32(p.k_scale + (size_t)(b * p.Hkv + hk) * nk + key_tile(j));
             const uint32_t s_addr = s_col + (uint32_t)(k & 1) * 128u;
             const uint32_t x_addr = xrow + (uint32_t)(k & 1) * 2048u;
             const bool diag = p.causal && (key_tile(j) == qi);
@@ -875,8 +891,7 @@ static inline baps_status attention_tc_launch(const void *q, const void *k, cons
     auto launch = [&](auto kernel, int sm) -> baps_status {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) != cudaSuccess)
             return BAPS_ERR_CUDA;
-        kernel<<<(unsigned)nblocks, kTcThreads, sm, stream>>>(mq, mk, mv, p);
-        return launch_status();
+        return launch_kernel(kernel, (unsigned)nblocks, kTcThreads, (size_t)sm, stream, mq, mk, mv, p);
     };
     constexpr int kE2E = BAPS_MODE_E2E_HIF8, kExact = BAPS_MODE_EXACT, kExp2m = BAPS_MODE_EXP2_HIF8;
     const bool b0l = p.b0_last != 0;

@@ -33,6 +33,37 @@ inline baps_status launch_status()
     return BAPS_OK;
 }
 
+// Programmatic dependent launch.  Every kernel of the library is launched with the attribute that lets it start
+// before the kernel ahead of it in the stream has ended, does what needs no caller memory (tables, barriers,
+// tensor memory), and waits for that kernel -- its completion, whatever it is -- before it touches any.  The wait
+// hands the pointer through, so that no load from it, not even one the compiler takes for invariant, can
+// move ahead of the wait.  The allow call is made by every CTA when it starts: the next kernel then comes in
+// as this one's last CTAs drain.
+__device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void await_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename T>
+__device__ __forceinline__ T *await_previous_kernel(T *p)
+{
+    asm volatile("griddepcontrol.wait;" : "+l"(p) :: "memory");
+    return p;
+}
+
+template <typename... P, typename... A>
+inline baps_status launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return BAPS_ERR_CUDA;
+    }
+    return launch_status();
+}
+
 inline bool have_device()
 {
     int dev = -1;

@@ -58,6 +58,7 @@ __device__ __forceinline__ uint32_t pack4_codes(float4 f, const uint8_t *s_tab)
 __global__ void __launch_bounds__(kEwThreads)
 hif8_encode_kernel(const float *__restrict__ x, uint8_t *__restrict__ codes, size_t n)
 {
+    allow_next_kernel();
     __shared__ __align__(16) uint8_t s_pack[8192];
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(g_encode_table);
@@ -65,6 +66,7 @@ hif8_encode_kernel(const float *__restrict__ x, uint8_t *__restrict__ codes, siz
         for (int i = threadIdx.x; i < 8192 / 16; i += kEwThreads) dst[i] = src[i];
     }
     __syncthreads();
+    x = await_previous_kernel(x);
     const size_t n4 = n / 4;
     const float4 *x4 = reinterpret_cast<const float4 *>(x);
     uint32_t *c4 = reinterpret_cast<uint32_t *>(codes);
@@ -95,6 +97,7 @@ hif8_encode_kernel(const float *__restrict__ x, uint8_t *__restrict__ codes, siz
 __global__ void __launch_bounds__(kEwThreads)
 hif8_decode_kernel(const uint8_t *__restrict__ codes, float *__restrict__ x, size_t n)
 {
+    allow_next_kernel();
     __shared__ __align__(16) uint32_t rep[128 * 32];
     for (int e2 = threadIdx.x; e2 < 128; e2 += kEwThreads) {
         const uint32_t lo = __float_as_uint(hif8_unpack((uint8_t)(2 * e2))) >> 16;
@@ -105,6 +108,7 @@ hif8_decode_kernel(const uint8_t *__restrict__ codes, float *__restrict__ x, siz
         for (int i = 0; i < 8; ++i) reinterpret_cast<uint4 *>(rep)[e2 * 8 + i] = w4;
     }
     __syncthreads();
+    codes = await_previous_kernel(codes);
     const int lane = threadIdx.x & 31;
     const uint8_t *lut = reinterpret_cast<const uint8_t *>(rep) + lane * 4;
     // codes 2k and 2k + 1 share the word k * 32 + lane
@@ -146,6 +150,7 @@ hif8_decode_kernel(const uint8_t *__restrict__ codes, float *__restrict__ x, siz
 __global__ void __launch_bounds__(kEwThreads)
 hif8_exp2_kernel(const uint8_t *__restrict__ t_codes, uint8_t *__restrict__ p_codes, size_t n)
 {
+    allow_next_kernel();
     __shared__ __align__(16) uint32_t rep[256 * 32];
     for (int e = threadIdx.x; e < 256; e += kEwThreads) {
         const uint32_t v = g_exp2_map[e];
@@ -154,6 +159,7 @@ hif8_exp2_kernel(const uint8_t *__restrict__ t_codes, uint8_t *__restrict__ p_co
         for (int i = 0; i < 8; ++i) reinterpret_cast<uint4 *>(rep)[e * 8 + i] = v4;
     }
     __syncthreads();
+    t_codes = await_previous_kernel(t_codes);
     const uint32_t *lut = rep + (threadIdx.x & 31);
     const size_t n16 = n / 16;
     const uint4 *t4 = reinterpret_cast<const uint4 *>(t_codes);

@@ -46,8 +46,7 @@ baps_status attention_f32_launch(const AttnF32Params &p, cudaStream_t st)
     const size_t sm = sizeof(float) * (size_t)L(p.D).total;
     if (set_smem(attention_f32_kernel<BLK>, sm) != BAPS_OK) return BAPS_ERR_CUDA;
     const dim3 grid((unsigned)(p.S / BLK) * kAfCluster, p.H, p.B);
-    attention_f32_kernel<BLK><<<grid, L::THREADS, sm, st>>>(p);
-    return launch_status();
+    return launch_kernel(attention_f32_kernel<BLK>, grid, L::THREADS, sm, st, p);
 }
 
 baps_status check_attention_common(const void *q, const void *k, const void *v, int B, int H,
@@ -200,8 +199,7 @@ baps_status baps_hif8_encode(const float *x, uint8_t *codes, size_t n, baps_stre
     const baps_status ts = ensure_ew_tables(as_stream(stream));
     if (ts != BAPS_OK) return ts;
     const size_t units = n / 4 / ((size_t)kEwThreads * kEwUnroll);
-    hif8_encode_kernel<<<ew_grid(units, num_sms()), kEwThreads, 0, as_stream(stream)>>>(x, codes, n);
-    return launch_status();
+    return launch_kernel(hif8_encode_kernel, ew_grid(units, num_sms()), kEwThreads, 0, as_stream(stream), x, codes, n);
 }
 
 baps_status baps_hif8_decode(const uint8_t *codes, float *x, size_t n, baps_stream stream)
@@ -211,8 +209,7 @@ baps_status baps_hif8_decode(const uint8_t *codes, float *x, size_t n, baps_stre
     if (!aligned16(x) || !aligned16(codes)) return BAPS_ERR_ALIGNMENT;
     if (!have_device()) return BAPS_ERR_CUDA;
     const size_t units = n / 16 / (size_t)kEwThreads;
-    hif8_decode_kernel<<<ew_grid(units, num_sms()), kEwThreads, 0, as_stream(stream)>>>(codes, x, n);
-    return launch_status();
+    return launch_kernel(hif8_decode_kernel, ew_grid(units, num_sms()), kEwThreads, 0, as_stream(stream), codes, x, n);
 }
 
 baps_status baps_exp2_hif8(const uint8_t *t_codes, uint8_t *p_codes, size_t n, baps_stream stream)
@@ -224,8 +221,7 @@ baps_status baps_exp2_hif8(const uint8_t *t_codes, uint8_t *p_codes, size_t n, b
     const baps_status ts = ensure_ew_tables(as_stream(stream));
     if (ts != BAPS_OK) return ts;
     const size_t units = n / 16 / ((size_t)kEwThreads * 2);
-    hif8_exp2_kernel<<<ew_grid(units, num_sms(), 8), kEwThreads, 0, as_stream(stream)>>>(t_codes, p_codes, n);
-    return launch_status();
+    return launch_kernel(hif8_exp2_kernel, ew_grid(units, num_sms(), 8), kEwThreads, 0, as_stream(stream), t_codes, p_codes, n);
 }
 
 baps_status baps_softmax_rows(const float *logits, float *probs, int64_t rows, int64_t cols,

@@ -303,7 +303,9 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t rep = sm100::smem_u32(s_rep) + (uint32_t)lane * 4u;
+    allow_next_kernel();
     fill_tables<CODES>(s_lut, s_rep, tid, nwarps * 32);
+    logits = await_previous_kernel(logits);
     if (tid == 0) {
         sm100::mbar_init(sm100::smem_u32(&s_full), 1);
         sm100::mbar_fence_init();
@@ -425,7 +427,9 @@ softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int6
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t rep = sm100::smem_u32(s_rep) + (uint32_t)lane * 4u;
+    allow_next_kernel();
     fill_tables<CODES>(s_lut, s_rep, tid, THREADS);
+    logits = await_previous_kernel(logits);
     if (tid == 0) {
         for (int i = 0; i < 3; ++i) sm100::mbar_init(sm100::smem_u32(&s_full[i]), 1);
         sm100::mbar_fence_init();
@@ -573,7 +577,9 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
     __shared__ __align__(16) uint32_t s_rep[(16 + kLutNegN) * 32];
     __shared__ float s_red_all[kMaxWarps];
     __shared__ float s_mfinal[15];
+    allow_next_kernel();
     fill_tables<CODES>(s_lut, s_rep, threadIdx.x, nt * ngroups);
+    logits = await_previous_kernel(logits);
     __syncthreads();
     const int grp = threadIdx.x / nt, tid = threadIdx.x % nt, lane = tid & 31, warp = tid >> 5;
     const uint32_t rep = sm100::smem_u32(s_rep) + (uint32_t)lane * 4u;
@@ -686,7 +692,9 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t rep = sm100::smem_u32(s_rep) + (uint32_t)lane * 4u;
     float2 *const s_blk = s_blk_all[warp];
+    allow_next_kernel();
     fill_tables<CODES>(s_lut, s_rep, tid, 512);
+    logits = await_previous_kernel(logits);
     __syncthreads();
     const int64_t step = (int64_t)gridDim.x * 16 * ROWS;
     for (int64_t row0 = ((int64_t)blockIdx.x * 16 + warp) * ROWS; row0 < rows; row0 += step) {
@@ -772,24 +780,21 @@ inline baps_status softmax_rows_codes_dispatch(const float *logits, uint8_t *cod
     };
     // (grids as in the float-output dispatch below: several times what is resident)
     const RowsOut out = {nullptr, codes, block_exp, row_d};
-    auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) {
+    auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) -> baps_status {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
             return BAPS_ERR_CUDA;
-        kernel<<<grid_for(ctas_per_sm), threads, dyn, st>>>(logits, out, rows, lambda, cols);
-        return BAPS_OK;
+        return launch_kernel(kernel, grid_for(ctas_per_sm), threads, (size_t)dyn, st, logits, out, rows, lambda, cols);
     };
     // a group per row: `threads` of them (or, other lengths, as few warps as hold the row, NV chunks each)
     auto group = [&](auto kernel, int threads, int max_threads, int ctas) {
         const int groups = max_threads / threads < 15 ? max_threads / threads : 15;
         const int64_t want = (rows + groups - 1) / groups, cap = (int64_t)num_sms * ctas;
-        kernel<<<(int)(want < cap ? want : cap), threads * groups, 0, st>>>(logits, out, rows, lambda, cols, threads);
-        return BAPS_OK;
+        return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), threads * groups, 0, st, logits, out, rows, lambda, cols, threads);
     };
     const int nch = cols / 128, t4 = (nch + 3) / 4 * 32, t8 = (nch + 7) / 8 * 32;
     auto warp_rows = [&](auto kernel, int rows_per_warp) {
         const int64_t want = (rows + 16 * rows_per_warp - 1) / (16 * rows_per_warp), cap = (int64_t)num_sms * 32;
-        kernel<<<(int)(want < cap ? want : cap), 512, 0, st>>>(logits, out, rows, lambda);
-        return BAPS_OK;
+        return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), 512, 0, st, logits, out, rows, lambda);
     };
     baps_status rc;
     switch (cols) {
@@ -820,8 +825,7 @@ inline baps_status softmax_rows_codes_dispatch(const float *logits, uint8_t *cod
         else rc = ring(softmax_rows_quarters_kernel<BK, true, false>, 1024, 196608, 2);
         break;
     }
-    if (rc != BAPS_OK) return rc;
-    return launch_status();
+    return rc;
 }
 
 // Launch the variant for the row length (see the head of this file).
@@ -834,11 +838,10 @@ inline baps_status softmax_rows_dispatch(const float *logits, float *probs, int6
         return (int)(rows < cap ? rows : cap);
     };
     const RowsOut out = {probs, nullptr, nullptr, nullptr};
-    auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) {
+    auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) -> baps_status {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
             return BAPS_ERR_CUDA;
-        kernel<<<grid_for(ctas_per_sm), threads, dyn, st>>>(logits, out, rows, lambda, cols);
-        return BAPS_OK;
+        return launch_kernel(kernel, grid_for(ctas_per_sm), threads, (size_t)dyn, st, logits, out, rows, lambda, cols);
     };
     // Grids: several times the CTAs that are resident at once (a few rows per CTA), so that the hardware
     // scheduler evens out the SMs; measured on 2^28 logits, a grid of exactly the resident CTAs -- each
@@ -851,14 +854,12 @@ inline baps_status softmax_rows_dispatch(const float *logits, float *probs, int6
     auto group = [&](auto kernel, int threads, int max_threads, int ctas) {
         const int groups = max_threads / threads < 15 ? max_threads / threads : 15;
         const int64_t want = (rows + groups - 1) / groups, cap = (int64_t)num_sms * ctas;
-        kernel<<<(int)(want < cap ? want : cap), threads * groups, 0, st>>>(logits, out, rows, lambda, cols, threads);
-        return BAPS_OK;
+        return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), threads * groups, 0, st, logits, out, rows, lambda, cols, threads);
     };
     const int nch = cols / 128, t4 = (nch + 3) / 4 * 32, t8 = (nch + 7) / 8 * 32;
     auto warp_rows = [&](auto kernel, int rows_per_warp) {
         const int64_t want = (rows + 16 * rows_per_warp - 1) / (16 * rows_per_warp), cap = (int64_t)num_sms * 32;
-        kernel<<<(int)(want < cap ? want : cap), 512, 0, st>>>(logits, out, rows, lambda);
-        return BAPS_OK;
+        return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), 512, 0, st, logits, out, rows, lambda);
     };
     baps_status rc;
     switch (cols) {
@@ -889,8 +890,7 @@ inline baps_status softmax_rows_dispatch(const float *logits, float *probs, int6
         else rc = ring(softmax_rows_quarters_kernel<BK, false, false>, 1024, 196608, 2);
         break;
     }
-    if (rc != BAPS_OK) return rc;
-    return launch_status();
+    return rc;
 }
 
 } // namespace baps
