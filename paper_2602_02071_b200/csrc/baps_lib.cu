@@ -199,7 +199,7 @@ baps_status baps_hif8_encode(const float *x, uint8_t *codes, size_t n, baps_stre
     const baps_status ts = ensure_ew_tables(as_stream(stream));
     if (ts != BAPS_OK) return ts;
     const size_t units = n / 4 / ((size_t)kEwThreads * kEwUnroll);
-    return launch_kernel(hif8_encode_kernel, ew_grid(units, num_sms()), kEwThreads, 0, as_stream(stream), x, codes, n);
+    return launch_kernel(hif8_encode_kernel, ew_grid(units, num_sms(), kEncodeIters), kEwThreads, 0, as_stream(stream), x, codes, n);
 }
 
 baps_status baps_hif8_decode(const uint8_t *codes, float *x, size_t n, baps_stream stream)
@@ -209,7 +209,7 @@ baps_status baps_hif8_decode(const uint8_t *codes, float *x, size_t n, baps_stre
     if (!aligned16(x) || !aligned16(codes)) return BAPS_ERR_ALIGNMENT;
     if (!have_device()) return BAPS_ERR_CUDA;
     const size_t units = n / 16 / (size_t)kEwThreads;
-    return launch_kernel(hif8_decode_kernel, ew_grid(units, num_sms()), kEwThreads, 0, as_stream(stream), codes, x, n);
+    return launch_kernel(hif8_decode_kernel, ew_grid(units, num_sms(), kDecodeIters), kEwThreads, 0, as_stream(stream), codes, x, n);
 }
 
 baps_status baps_exp2_hif8(const uint8_t *t_codes, uint8_t *p_codes, size_t n, baps_stream stream)
@@ -221,7 +221,7 @@ baps_status baps_exp2_hif8(const uint8_t *t_codes, uint8_t *p_codes, size_t n, b
     const baps_status ts = ensure_ew_tables(as_stream(stream));
     if (ts != BAPS_OK) return ts;
     const size_t units = n / 16 / ((size_t)kEwThreads * 2);
-    return launch_kernel(hif8_exp2_kernel, ew_grid(units, num_sms(), 8), kEwThreads, 0, as_stream(stream), t_codes, p_codes, n);
+    return launch_kernel(hif8_exp2_kernel, ew_grid(units, num_sms(), kExp2Iters), kEwThreads, 0, as_stream(stream), t_codes, p_codes, n);
 }
 
 baps_status baps_softmax_rows(const float *logits, float *probs, int64_t rows, int64_t cols,
