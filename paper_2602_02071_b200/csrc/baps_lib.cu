@@ -5,7 +5,7 @@
 #include "baps_elementwise.cuh"
 #include "baps_softmax_rows.cuh"
 #include "baps_attention_f32.cuh"
-#include "baps_attention_tc.cuh"
+#include "baps_attention_launch.cuh"
 
 #include <cmath>
 #include <mutex>
