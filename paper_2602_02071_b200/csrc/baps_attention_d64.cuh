@@ -18,7 +18,7 @@
 // attention_tc_kernel; only the row sum is added up in another order (two partial sums per row, not four).
 // Measured against that kernel with two query tiles per CTA (heads x tokens): 512 x 1024 bidirectional 351 -> 330 us,
 // 64 x 8192 causal 1233 -> 1101, 24 x 2048 causal 46.2 -> 42.8 on unit-Gaussian inputs; with a per-token key bias
-// (more restarts and positive T) 512 x 1024 342 -> 342.  Small grids keep that kernel (two_ctas_per_sm).
+// (more restarts and positive T) 512 x 1024 342 -> 313.  Small grids keep that kernel (two_ctas_per_sm).
 #pragma once
 #include "baps_attention_tc.cuh"
 
@@ -61,14 +61,8 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
     allow_next_kernel();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // ---- work assignment: heavy (late) query tiles first; the query heads of one kv head adjacent
-    const int gsz = p.H / p.Hkv;
-    int idx = blockIdx.x;
-    const int gi = idx % gsz; idx /= gsz;
-    const int hk = idx % p.Hkv; idx /= p.Hkv;
-    const int b = idx % p.B; idx /= p.B;
-    const int qi = p.nq - 1 - idx;
-    const int h = hk * gsz + gi;
+    const WorkItem item = work_item(p, blockIdx.x);
+    const int qi = item.tile, hk = item.hk, b = item.b, h = item.h;
     const int J = p.causal ? qi + 1 : p.nq;               // number of key tiles
     const int q_row0 = (b * p.H + h) * p.S + qi * 128;    // row in the [B*H*S, D] view
     const int kv_row0 = (b * p.Hkv + hk) * p.S;

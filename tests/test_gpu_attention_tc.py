@@ -276,3 +276,20 @@ def test_two_ctas_per_sm_d64_against_the_checker(causal, lam):
     gate_attention(st.out_f32[at].cpu().numpy(), ref, what=f"d64 causal={causal} lam={lam}")
     same = (st.row_m[at].cpu().numpy().reshape(ref.row_m.shape) == ref.row_m)
     assert same[ref.row_margin > EPS_REL].all()
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("B,Hkv,g,D", [(23, 7, 1, 64), (9, 5, 3, 128), (301, 1, 2, 128)])
+def test_chunks_of_heads_cover_every_tile(B, Hkv, g, D, causal):
+    """Head counts that leave the last chunk of kv heads ragged: every (batch, head) as when run alone."""
+    S = 2048 if D == 128 and B < 100 else 1024
+    gen = torch.Generator(device="cuda"); gen.manual_seed(B)
+    q, k, v = (torch.randn(B, h, S, D, device="cuda", generator=gen).bfloat16() for h in (Hkv * g, Hkv, Hkv))
+    out = torch.full_like(q, float("nan"))
+    binding.baps_attention_fwd(q, k, v, causal=causal, out=out)
+    assert not torch.isnan(out).any()
+    for b, h in ((0, 0), (B // 2, Hkv - 1), (B - 1, 0), (B - 1, Hkv - 1)):
+        alone = binding.baps_attention_fwd(q[b:b + 1, h * g:(h + 1) * g].contiguous(), k[b:b + 1, h:h + 1].contiguous(),
+                                           v[b:b + 1, h:h + 1].contiguous(), causal=causal)
+        # (D = 64: the lone head takes the other kernel, whose row sum is added up in another order)
+        assert torch.allclose(out[b, h * g:(h + 1) * g].float(), alone[0].float(), rtol=2.0 ** -7, atol=0)
