@@ -61,7 +61,7 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
     allow_next_kernel();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    const WorkItem item = work_item(p, blockIdx.x);
+    const WorkItem item = work_item(p.H, p.Hkv, p.npairs, p.chunks, blockIdx.x);
     const int qi = item.tile, hk = item.hk, b = item.b, h = item.h;
     const int J = p.causal ? qi + 1 : p.nq;               // number of key tiles
     const int q_row0 = (b * p.H + h) * p.S + qi * 128;    // row in the [B*H*S, D] view

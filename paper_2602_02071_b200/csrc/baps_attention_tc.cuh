@@ -34,6 +34,7 @@
 #include "baps_hif8.cuh"
 #include "baps_sm100.cuh"
 #include "baps_tables.cuh"
+#include "baps_tile_order.cuh"
 
 namespace baps {
 
@@ -54,29 +55,8 @@ struct AttnTcParams {
     const float *k_scale;     // dequantisation scales (powers of two); null otherwise
     float c;                  // log2(e) * scale
     int nq, npairs;           // query tiles; work items per head (pairs of query tiles, or single tiles)
-    int chunk;                // kv heads (of all batches) worked on together, see work_item
+    KvChunks chunks;          // kv heads (of all batches) worked on together, see work_item
 };
-
-// Which tile of which head a CTA works on.  The kv heads are taken in chunks (p.chunk of the B * Hkv) whose K and
-// V together stay in L2 while their query tiles pass; within a chunk the heavy (late) query tiles come first and the
-// query heads of one kv head are adjacent.  (Taken all at once, 512 heads x 1024 tokens of D = 64 -- 134 MB of K and
-// V -- were read from HBM again for every query tile.)
-struct WorkItem { int tile, h, hk, b; };
-__device__ __forceinline__ WorkItem work_item(const AttnTcParams &p, int idx)
-{
-    const int gsz = p.H / p.Hkv, per_chunk = p.chunk * gsz * p.npairs;
-    const int first = idx / per_chunk * p.chunk, n = min(p.chunk, p.B * p.Hkv - first);
-    idx %= per_chunk;
-    const int gi = idx % gsz;
-    idx /= gsz;
-    const int kv = first + idx % n;
-    WorkItem w;
-    w.tile = p.npairs - 1 - idx / n;
-    w.hk = kv % p.Hkv;
-    w.b = kv / p.Hkv;
-    w.h = w.hk * gsz + gi;
-    return w;
-}
 
 constexpr int kTcThreads = 640;
 constexpr int kTcSoftmaxWarps = 16;
@@ -294,7 +274,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     allow_next_kernel();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    const WorkItem item = work_item(p, blockIdx.x);
+    const WorkItem item = work_item(p.H, p.Hkv, p.npairs, p.chunks, blockIdx.x);
     const int pair = item.tile, hk = item.hk, b = item.b, h = item.h;
     const int nk = p.S / 128;
     // With B0 = {first, last} the key tiles are visited in the order 0, last, 1, ..., last - 1, and
