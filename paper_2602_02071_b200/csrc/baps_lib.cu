@@ -28,25 +28,24 @@ int num_sms()
     return cached[dev];
 }
 
-template <typename K>
-baps_status set_smem(K kernel, size_t bytes)
-{
-    if (bytes > 48 * 1024) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
-            cudaSuccess)
-            return BAPS_ERR_CUDA;
-    }
-    return BAPS_OK;
-}
-
 template <int BLK>
 baps_status attention_f32_launch(const AttnF32Params &p, cudaStream_t st)
 {
     using L = AfLayout<BLK>;
-    const size_t sm = sizeof(float) * (size_t)L(p.D).total;
-    if (set_smem(attention_f32_kernel<BLK>, sm) != BAPS_OK) return BAPS_ERR_CUDA;
+    // the limit is state of the kernel, which other threads may be launching with other head sizes: always the
+    // largest head's
+    const int most = (int)sizeof(float) * L(128).total;
+    if (cudaFuncSetAttribute(attention_f32_kernel<BLK>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
+        return BAPS_ERR_CUDA;
     const dim3 grid((unsigned)(p.S / BLK) * kAfCluster, p.H, p.B);
-    return launch_kernel(attention_f32_kernel<BLK>, grid, L::THREADS, sm, st, p);
+    return launch_kernel(attention_f32_kernel<BLK>, grid, L::THREADS, sizeof(float) * (size_t)L(p.D).total, st, p);
+}
+
+template <bool CODES>
+baps_status softmax_rows_launch(const RowsOut &out, const float *logits, int64_t rows, int64_t cols, int block_k, baps_stream stream)
+{
+    return block_k == 64 ? softmax_rows_dispatch<64, CODES>(logits, out, rows, (int)cols, 1, num_sms(), as_stream(stream))
+                         : softmax_rows_dispatch<128, CODES>(logits, out, rows, (int)cols, 1, num_sms(), as_stream(stream));
 }
 
 baps_status check_attention_common(const void *q, const void *k, const void *v, int B, int H,
@@ -234,9 +233,7 @@ baps_status baps_softmax_rows(const float *logits, float *probs, int64_t rows, i
         return BAPS_ERR_UNSUPPORTED;
     if (!aligned16(logits) || !aligned16(probs)) return BAPS_ERR_ALIGNMENT;
     if (!have_device()) return BAPS_ERR_CUDA;
-    if (block_k == 64)
-        return softmax_rows_dispatch<64>(logits, probs, rows, (int)cols, 1, num_sms(), as_stream(stream));
-    return softmax_rows_dispatch<128>(logits, probs, rows, (int)cols, 1, num_sms(), as_stream(stream));
+    return softmax_rows_launch<false>({probs, nullptr, nullptr, nullptr}, logits, rows, cols, block_k, stream);
 }
 
 baps_status baps_softmax_rows_codes(const float *logits, uint8_t *codes, int32_t *block_exp, float *row_d,
@@ -248,9 +245,7 @@ baps_status baps_softmax_rows_codes(const float *logits, uint8_t *codes, int32_t
     if ((block_k != 64 && block_k != 128) || cols % 128 != 0 || cols > 65536) return BAPS_ERR_UNSUPPORTED;
     if (!aligned16(logits) || !aligned16(codes) || !aligned4(block_exp) || !aligned4(row_d)) return BAPS_ERR_ALIGNMENT;
     if (!have_device()) return BAPS_ERR_CUDA;
-    if (block_k == 64)
-        return softmax_rows_codes_dispatch<64>(logits, codes, block_exp, row_d, rows, (int)cols, 1, num_sms(), as_stream(stream));
-    return softmax_rows_codes_dispatch<128>(logits, codes, block_exp, row_d, rows, (int)cols, 1, num_sms(), as_stream(stream));
+    return softmax_rows_launch<true>({nullptr, codes, block_exp, row_d}, logits, rows, cols, block_k, stream);
 }
 
 baps_status baps_attention_fwd_ex(const void *q, const void *k, const void *v, void *out,

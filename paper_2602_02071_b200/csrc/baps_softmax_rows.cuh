@@ -770,127 +770,63 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
 // The table entries carry value and code in one word: a HiF8 value has at most four significant mantissa
 // bits, so the low byte of its fp32 pattern is free for the code.
 
-template <int BK>
-inline baps_status softmax_rows_codes_dispatch(const float *logits, uint8_t *codes, int32_t *block_exp, float *row_d,
-                                               int64_t rows, int cols, int lambda, int num_sms, cudaStream_t st)
-{
-    auto grid_for = [&](int ctas_per_sm) {
-        const int64_t cap = (int64_t)num_sms * ctas_per_sm;
-        return (int)(rows < cap ? rows : cap);
-    };
-    // (grids as in the float-output dispatch below: several times what is resident)
-    const RowsOut out = {nullptr, codes, block_exp, row_d};
-    auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) -> baps_status {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
-            return BAPS_ERR_CUDA;
-        return launch_kernel(kernel, grid_for(ctas_per_sm), threads, (size_t)dyn, st, logits, out, rows, lambda, cols);
-    };
-    // a group per row: `threads` of them (or, other lengths, as few warps as hold the row, NV chunks each)
-    auto group = [&](auto kernel, int threads, int max_threads, int ctas) {
-        const int groups = max_threads / threads < 15 ? max_threads / threads : 15;
-        const int64_t want = (rows + groups - 1) / groups, cap = (int64_t)num_sms * ctas;
-        return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), threads * groups, 0, st, logits, out, rows, lambda, cols, threads);
-    };
-    const int nch = cols / 128, t4 = (nch + 3) / 4 * 32, t8 = (nch + 7) / 8 * 32;
-    auto warp_rows = [&](auto kernel, int rows_per_warp) {
-        const int64_t want = (rows + 16 * rows_per_warp - 1) / (16 * rows_per_warp), cap = (int64_t)num_sms * 32;
-        return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), 512, 0, st, logits, out, rows, lambda);
-    };
-    baps_status rc;
-    switch (cols) {
-    case 128:   rc = warp_rows(softmax_rows_warp_kernel<BK, 1, 4, true>, 4); break;
-    case 256:   rc = warp_rows(softmax_rows_warp_kernel<BK, 2, 4, true>, 4); break;
-    case 384:   rc = warp_rows(softmax_rows_warp_kernel<BK, 3, 2, true>, 2); break;
-    case 512:   rc = warp_rows(softmax_rows_warp_kernel<BK, 4, 2, true>, 2); break;
-    case 640:   rc = warp_rows(softmax_rows_warp_kernel<BK, 5, 1, true>, 1); break;
-    case 768:   rc = warp_rows(softmax_rows_warp_kernel<BK, 6, 1, true>, 1); break;
-    case 896:   rc = warp_rows(softmax_rows_warp_kernel<BK, 7, 1, true>, 1); break;
-    case 1024:  rc = warp_rows(softmax_rows_warp_kernel<BK, 8, 1, true>, 1); break;
-    case 1152:  rc = warp_rows(softmax_rows_warp_kernel<BK, 9, 1, true>, 1); break;
-    case 2048:  rc = group(softmax_rows_group_kernel<BK, 128, 4, 4, true, true>, 128, 512, 16); break;
-    case 4096:  rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, true, true, true>, 256, 1024, 4); break;
-    case 8192:  rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, true, false>, 256, 1024, 4); break;
-    case 16384: rc = ring(softmax_rows_ring_kernel<BK, 512, true, true>, 512, 65536, 2); break;
-    case 32768: rc = ring(softmax_rows_ring_kernel<BK, 1024, true>, 1024, 131072, 2); break;
-    case 65536: rc = ring(softmax_rows_quarters_kernel<BK, true>, 1024, 196608, 2); break;
-    default:
-        // Other lengths: as few warps per row as hold it, NV consecutive chunks of 128 columns each (every test
-        // for the end of the row is the same for a whole warp).  Four chunks per warp and the next row's loads
-        // in flight up to 1536 columns, eight from there on (2^27 logits, float / 8-bit output: 1536 columns 176 /
-        // 161 us against 179 / 170, 1920 columns 183 / 183 against 176 / 144).
-        if (cols <= 1536) rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, true, true, true, false>, t4, 1024, 4);
-        else if (cols < 8192) rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, true, false, true, false>, t8, 1024, 4);
-        else if (cols < 16384) rc = ring(softmax_rows_ring_kernel<BK, 512, true, true, false>, t8, cols * 4, 4);
-        else if (cols < 32768) rc = ring(softmax_rows_ring_kernel<BK, 1024, true, true, false>, t8, cols * 4, 2);
-        else rc = ring(softmax_rows_quarters_kernel<BK, true, false>, 1024, 196608, 2);
-        break;
-    }
-    return rc;
-}
-
 // Launch the variant for the row length (see the head of this file).
-template <int BK>
-inline baps_status softmax_rows_dispatch(const float *logits, float *probs, int64_t rows, int cols, int lambda,
-                                  int num_sms, cudaStream_t st)
+// Grids: several times the CTAs that are resident at once (a few rows per CTA), so that the hardware
+// scheduler evens out the SMs; measured on 2^28 logits, a grid of exactly the resident CTAs -- each
+// with a fixed share of the rows -- loses 5 to 10 % to the slowest SM.
+// Up to 8K columns the rows are register-resident and several rows share a CTA and its tables
+// (softmax_rows_group_kernel: 16 or 32 elements per thread); up to 1152 a warp per row needs no barrier at
+// all.  At 16K and 32K only one or two CTAs fit an SM, and the ring lets the next row's read overlap
+// the current row's passes.
+template <int BK, bool CODES>
+inline baps_status softmax_rows_dispatch(const float *logits, const RowsOut &out, int64_t rows, int cols, int lambda,
+                                         int num_sms, cudaStream_t st)
 {
-    auto grid_for = [&](int ctas_per_sm) {
-        const int64_t cap = (int64_t)num_sms * ctas_per_sm;
-        return (int)(rows < cap ? rows : cap);
-    };
-    const RowsOut out = {probs, nullptr, nullptr, nullptr};
-    auto ring = [&](auto kernel, int threads, int dyn, int ctas_per_sm) -> baps_status {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
+    // a CTA per row.  The kernel's shared memory limit is state of the kernel, which other threads may be launching
+    // with other row lengths: it is always set to the most the instance takes (kernel_most), the launch asks for `dyn`.
+    auto ring = [&](auto kernel, int threads, int dyn, int kernel_most, int ctas_per_sm) -> baps_status {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kernel_most) != cudaSuccess)
             return BAPS_ERR_CUDA;
-        return launch_kernel(kernel, grid_for(ctas_per_sm), threads, (size_t)dyn, st, logits, out, rows, lambda, cols);
+        const int64_t cap = (int64_t)num_sms * ctas_per_sm;
+        return launch_kernel(kernel, (unsigned)(rows < cap ? rows : cap), threads, (size_t)dyn, st, logits, out, rows, lambda, cols);
     };
-    // Grids: several times the CTAs that are resident at once (a few rows per CTA), so that the hardware
-    // scheduler evens out the SMs; measured on 2^28 logits, a grid of exactly the resident CTAs -- each
-    // with a fixed share of the rows -- loses 5 to 10 % to the slowest SM.
-    // Up to 8K columns the rows are register-resident and several rows share a CTA and its tables
-    // (softmax_rows_group_kernel: 16 or 32 elements per thread); at 1K a warp per row needs no barrier at
-    // all.  At 16K and 32K only one or two CTAs fit an SM, and the ring lets the next row's read overlap
-    // the current row's passes.
     // a group per row: `threads` of them (or, other lengths, as few warps as hold the row, NV chunks each)
     auto group = [&](auto kernel, int threads, int max_threads, int ctas) {
         const int groups = max_threads / threads < 15 ? max_threads / threads : 15;
         const int64_t want = (rows + groups - 1) / groups, cap = (int64_t)num_sms * ctas;
         return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), threads * groups, 0, st, logits, out, rows, lambda, cols, threads);
     };
-    const int nch = cols / 128, t4 = (nch + 3) / 4 * 32, t8 = (nch + 7) / 8 * 32;
     auto warp_rows = [&](auto kernel, int rows_per_warp) {
         const int64_t want = (rows + 16 * rows_per_warp - 1) / (16 * rows_per_warp), cap = (int64_t)num_sms * 32;
         return launch_kernel(kernel, (unsigned)(want < cap ? want : cap), 512, 0, st, logits, out, rows, lambda);
     };
-    baps_status rc;
+    const int nch = cols / 128, t4 = (nch + 3) / 4 * 32, t8 = (nch + 7) / 8 * 32;
     switch (cols) {
-    case 128:   rc = warp_rows(softmax_rows_warp_kernel<BK, 1, 4, false>, 4); break;
-    case 256:   rc = warp_rows(softmax_rows_warp_kernel<BK, 2, 4, false>, 4); break;
-    case 384:   rc = warp_rows(softmax_rows_warp_kernel<BK, 3, 2, false>, 2); break;
-    case 512:   rc = warp_rows(softmax_rows_warp_kernel<BK, 4, 2, false>, 2); break;
-    case 640:   rc = warp_rows(softmax_rows_warp_kernel<BK, 5, 1, false>, 1); break;
-    case 768:   rc = warp_rows(softmax_rows_warp_kernel<BK, 6, 1, false>, 1); break;
-    case 896:   rc = warp_rows(softmax_rows_warp_kernel<BK, 7, 1, false>, 1); break;
-    case 1024:  rc = warp_rows(softmax_rows_warp_kernel<BK, 8, 1, false>, 1); break;
-    case 1152:  rc = warp_rows(softmax_rows_warp_kernel<BK, 9, 1, false>, 1); break;
-    case 2048:  rc = group(softmax_rows_group_kernel<BK, 128, 4, 4, false, true>, 128, 512, 16); break;
-    case 4096:  rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, false, true, false>, 256, 1024, 4); break;
-    case 8192:  rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, false, false>, 256, 1024, 4); break;
-    case 16384: rc = ring(softmax_rows_ring_kernel<BK, 512, false, false>, 512, 65536, 2); break;
-    case 32768: rc = ring(softmax_rows_ring_kernel<BK, 1024, false>, 1024, 131072, 2); break;
-    case 65536: rc = ring(softmax_rows_quarters_kernel<BK, false>, 1024, 196608, 2); break;
-    default:
-        // Other lengths: as few warps per row as hold it, NV consecutive chunks of 128 columns each (every test
-        // for the end of the row is the same for a whole warp).  Four chunks per warp and the next row's loads
-        // in flight up to 1536 columns, eight from there on (2^27 logits, float / 8-bit output: 1536 columns 176 /
-        // 161 us against 179 / 170, 1920 columns 183 / 183 against 176 / 144).
-        if (cols <= 1536) rc = group(softmax_rows_group_kernel<BK, 256, 4, 4, false, true, true, false>, t4, 1024, 4);
-        else if (cols < 8192) rc = group(softmax_rows_group_kernel<BK, 256, 8, 4, false, false, true, false>, t8, 1024, 4);
-        else if (cols < 16384) rc = ring(softmax_rows_ring_kernel<BK, 512, false, true, false>, t8, cols * 4, 4);
-        else if (cols < 32768) rc = ring(softmax_rows_ring_kernel<BK, 1024, false, true, false>, t8, cols * 4, 2);
-        else rc = ring(softmax_rows_quarters_kernel<BK, false, false>, 1024, 196608, 2);
-        break;
+    case 128:   return warp_rows(softmax_rows_warp_kernel<BK, 1, 4, CODES>, 4);
+    case 256:   return warp_rows(softmax_rows_warp_kernel<BK, 2, 4, CODES>, 4);
+    case 384:   return warp_rows(softmax_rows_warp_kernel<BK, 3, 2, CODES>, 2);
+    case 512:   return warp_rows(softmax_rows_warp_kernel<BK, 4, 2, CODES>, 2);
+    case 640:   return warp_rows(softmax_rows_warp_kernel<BK, 5, 1, CODES>, 1);
+    case 768:   return warp_rows(softmax_rows_warp_kernel<BK, 6, 1, CODES>, 1);
+    case 896:   return warp_rows(softmax_rows_warp_kernel<BK, 7, 1, CODES>, 1);
+    case 1024:  return warp_rows(softmax_rows_warp_kernel<BK, 8, 1, CODES>, 1);
+    case 1152:  return warp_rows(softmax_rows_warp_kernel<BK, 9, 1, CODES>, 1);
+    case 2048:  return group(softmax_rows_group_kernel<BK, 128, 4, 4, CODES, true>, 128, 512, 16);
+    case 4096:  return group(softmax_rows_group_kernel<BK, 256, 4, 4, CODES, true, CODES>, 256, 1024, 4);
+    case 8192:  return group(softmax_rows_group_kernel<BK, 256, 8, 4, CODES, false>, 256, 1024, 4);
+    case 16384: return ring(softmax_rows_ring_kernel<BK, 512, CODES, CODES>, 512, 65536, 65536, 2);
+    case 32768: return ring(softmax_rows_ring_kernel<BK, 1024, CODES>, 1024, 131072, 131072, 2);
+    case 65536: return ring(softmax_rows_quarters_kernel<BK, CODES>, 1024, 196608, 196608, 2);
     }
-    return rc;
+    // Other lengths: as few warps per row as hold it, NV consecutive chunks of 128 columns each (every test
+    // for the end of the row is the same for a whole warp).  Four chunks per warp and the next row's loads
+    // in flight up to 1536 columns, eight from there on (2^27 logits, float / 8-bit output: 1536 columns 176 /
+    // 161 us against 179 / 170, 1920 columns 183 / 183 against 176 / 144).
+    if (cols <= 1536) return group(softmax_rows_group_kernel<BK, 256, 4, 4, CODES, true, true, false>, t4, 1024, 4);
+    if (cols < 8192) return group(softmax_rows_group_kernel<BK, 256, 8, 4, CODES, false, true, false>, t8, 1024, 4);
+    if (cols < 16384) return ring(softmax_rows_ring_kernel<BK, 512, CODES, true, false>, t8, cols * 4, 65536, 4);
+    if (cols < 32768) return ring(softmax_rows_ring_kernel<BK, 1024, CODES, true, false>, t8, cols * 4, 131072, 2);
+    return ring(softmax_rows_quarters_kernel<BK, CODES, false>, 1024, 196608, 196608, 2);
 }
 
 } // namespace baps
