@@ -439,6 +439,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
             auto wait_all = [&](uint32_t bar_addr, uint32_t parity, int code) -> bool {
                 return __all_sync(0xffffffffu, mbar_wait(bar_addr, parity, s_abort, &g_async_status, code));
             };
+            // (the limit of the first wait starts when the kernel ahead has ended, however long that takes; with kEarly
+            // the producer has waited for it before the CTA-wide barrier)
+            if constexpr (!kEarly) await_previous_kernel();
             bool ok = wait_all(bar(BQ), 0, 0x200);
             int k_ready = -1, v_ready = -1;      // key / value tiles whose arrival has been awaited
             auto await_k = [&](int j) -> bool {

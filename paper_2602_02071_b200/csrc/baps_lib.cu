@@ -154,6 +154,21 @@ int baps_test_skip_kv_load(int l)
 {
     return cudaMemcpyToSymbol(g_test_skip_load, &l, sizeof(int)) == cudaSuccess ? 0 : -1;
 }
+
+// Test build only: one block that lets the next kernel start at once and keeps the stream busy for `us`
+// microseconds (20 ms at most).
+static __global__ void test_busy_kernel(uint64_t ns)
+{
+    allow_next_kernel();
+    const uint64_t t0 = sm100::globaltimer_ns();
+    for (int i = 0; i < 1000000 && sm100::globaltimer_ns() - t0 < ns; ++i) __nanosleep(1000);
+}
+int baps_test_keep_busy(int us, baps_stream stream)
+{
+    if (us < 0 || us > 20000) return -1;
+    test_busy_kernel<<<1, 32, 0, as_stream(stream)>>>((uint64_t)us * 1000);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
 #endif
 
 baps_status baps_poll_async_error(baps_stream stream)
