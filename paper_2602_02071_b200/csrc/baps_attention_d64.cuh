@@ -58,7 +58,6 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::kMiscOff);
     volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L::kMiscOff + 4);
 
-    allow_next_kernel();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     const WorkItem item = work_item(p.H, p.Hkv, p.npairs, p.chunks, blockIdx.x);
@@ -93,7 +92,13 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
         }
         __syncwarp();
     } else if (warp == 9) {
+        // The allocation waits, without a limit, for tensor memory that another CTA on the SM holds.  So none is taken
+        // while a kernel ahead may still have to take its own, and the next kernel starts only when every CTA of this
+        // one has its share: no two can hold what the other waits for.  (attention_tc_kernel need not care: its CTA takes
+        // 61440 of the SM's 65536 registers, and nothing that uses tensor memory fits beside it.)
+        await_previous_kernel();
         tmem_alloc(smem_u32(s_tmem), 256); tmem_relinquish();
+        allow_next_kernel();
         if (lane == 0) { tma_prefetch_desc(&mq); tma_prefetch_desc(&mk); tma_prefetch_desc(&mv); }
     } else if (warp < kD64SoftmaxWarps) {
         float4 *rep = reinterpret_cast<float4 *>(smem + L::kLutRepOff);

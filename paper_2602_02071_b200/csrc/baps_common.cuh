@@ -37,8 +37,8 @@ inline baps_status launch_status()
 // before the kernel ahead of it in the stream has ended, does what needs no caller memory (tables, barriers,
 // tensor memory), and waits for that kernel -- its completion, whatever it is -- before it touches any.  The wait
 // hands the pointer through, so that no load from it, not even one the compiler takes for invariant, can
-// move ahead of the wait.  The allow call is made by every CTA when it starts: the next kernel then comes in
-// as this one's last CTAs drain.
+// move ahead of the wait.  The allow call is made by every CTA when it starts (attention_d64_kernel: when it has its
+// tensor memory): the next kernel then comes in as this one's last CTAs drain.
 __device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void await_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename T>
