@@ -124,7 +124,7 @@ attention_f32_kernel(const AttnF32Params p)
     fetch(s_K, lay.ks, kh);
     for (int i = tid; i < R * lay.Dp; i += THREADS) {
         const int r = i / lay.Dp, d = i % lay.Dp;
-        s_Q[r * lay.qs + d] = d < D ? (double)__ldg(qh + (size_t)(i0 + r) * D + d) : 0.0;
+        s_Q[r * lay.qs + d] = d < D ? (double)qh[(size_t)(i0 + r) * D + d] : 0.0;
     }
     if (lay.Dp > D)                                          // the copies never touch the padding
         for (int i = tid; i < BLK * (lay.Dp - D); i += THREADS)

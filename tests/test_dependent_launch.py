@@ -41,3 +41,9 @@ def test_tensor_memory_is_taken_between_the_kernel_ahead_and_the_next_one():
     assert body.index("await_previous_kernel()", role) < alloc < body.index("allow_next_kernel()")
     assert "__launch_bounds__(kTcThreads, 1)" in CODE["baps_attention_tc.cuh"]
     assert re.search(r"kTcThreads = 640;", CODE["baps_attention_tc.cuh"])
+
+
+def test_no_load_asks_for_data_that_never_changes():
+    """ld.global.nc (__ldg) may be served from data read before the kernel ahead wrote it."""
+    for name, code in CODE.items():
+        assert "__ldg(" not in code and "ld.global.nc" not in code, name
