@@ -32,13 +32,15 @@ template <int BLK>
 baps_status attention_f32_launch(const AttnF32Params &p, cudaStream_t st)
 {
     using L = AfLayout<BLK>;
-    // the limit is state of the kernel, which other threads may be launching with other head sizes: always the
-    // largest head's
+    // the limit is state of the kernel, which other threads may be launching with other head sizes: never anything but
+    // the largest head's (not set at all where the default does: 0.4 us of an 8.5 us call)
+    const size_t smem = sizeof(float) * (size_t)L(p.D).total;
     const int most = (int)sizeof(float) * L(128).total;
-    if (cudaFuncSetAttribute(attention_f32_kernel<BLK>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(attention_f32_kernel<BLK>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
         return BAPS_ERR_CUDA;
     const dim3 grid((unsigned)(p.S / BLK) * kAfCluster, p.H, p.B);
-    return launch_kernel(attention_f32_kernel<BLK>, grid, L::THREADS, sizeof(float) * (size_t)L(p.D).total, st, p);
+    return launch_kernel(attention_f32_kernel<BLK>, grid, L::THREADS, smem, st, p);
 }
 
 template <bool CODES>
