@@ -24,10 +24,7 @@
 
 namespace baps {
 
-constexpr int kD64Threads = 384, kD64SoftmaxWarps = 8;
-// Registers: the pool is what a CTA got at launch, 384 x 80 (two CTAs per SM).
-constexpr int kD64RegsFew = 32, kD64RegsMany = 104;
-static_assert(128 * kD64RegsFew + 256 * kD64RegsMany <= kD64Threads * 80, "within what the CTA got at launch");
+constexpr int kD64Threads = kD64Split.threads, kD64SoftmaxWarps = kD64Split.many_threads / 32;
 
 struct D64Layout {
     static constexpr int kTileBytes = 128 * 64 * 2, kStages = 4;
@@ -117,7 +114,7 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
     const uint32_t tmem = *s_tmem;                        // scores | weights (+ 128) | O~ (+ 192)
 
     if (warp >= kD64SoftmaxWarps) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kD64RegsFew));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kD64Split.few));
         if (warp == 8) {
             // ======================= TMA producer ==================================================
             if (lane == 0) {
@@ -184,7 +181,7 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
             }
         }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kD64RegsMany));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kD64Split.many));
         // ======================= softmax warps ==================================================
         await_previous_kernel();
         const int q4 = warp & 3;                 // TMEM lane quarter: rows 32 q4 .. 32 q4 + 31

@@ -32,6 +32,7 @@
 #include <cuda_bf16.h>
 #include "baps_common.cuh"
 #include "baps_hif8.cuh"
+#include "baps_register_split.cuh"
 #include "baps_sm100.cuh"
 #include "baps_tables.cuh"
 #include "baps_tile_order.cuh"
@@ -58,8 +59,8 @@ struct AttnTcParams {
     KvChunks chunks;          // kv heads (of all batches) worked on together, see work_item
 };
 
-constexpr int kTcThreads = 640;
-constexpr int kTcSoftmaxWarps = 16;
+constexpr int kTcThreads = kTcSplit.threads;
+constexpr int kTcSoftmaxWarps = kTcSplit.many_threads / 32;
 constexpr int kLutRepEntries = 16 + kLutNegN;              // keys 0 .. 192, 32 copies each
 constexpr int kLutRepBytes = kLutRepEntries * 128;
 
@@ -376,11 +377,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     const uint32_t tmem = *s_tmem;
 
     // Register budget: the fifth warpgroup (producer, MMA issuer, two idle warps) needs few
-    // registers and hands part of its share to the sixteen softmax warps.  The pool is what the
-    // CTA got at launch (640 x 96): 128 x 64 + 512 x 104 = 61440 uses it exactly; asking for more
-    // than the pool holds would block forever.
+    // registers and hands part of its share to the sixteen softmax warps (kTcSplit).
     if (warp >= kTcSoftmaxWarps) {
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kTcSplit.few));
       if (warp == 16) {
         // ======================= TMA producer ==================================================
         if (lane == 0) {
@@ -533,7 +532,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
         }
       }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kTcSplit.many));
         // ======================= softmax warps ==================================================
         // (kEarly: the tables were filled before the CTA-wide barrier, while a kernel ahead was still draining)
         if constexpr (!kEarly) {

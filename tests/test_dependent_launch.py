@@ -40,7 +40,8 @@ def test_tensor_memory_is_taken_between_the_kernel_ahead_and_the_next_one():
     role = body.rindex("else if (warp == 9)", 0, alloc)
     assert body.index("await_previous_kernel()", role) < alloc < body.index("allow_next_kernel()")
     assert "__launch_bounds__(kTcThreads, 1)" in CODE["baps_attention_tc.cuh"]
-    assert re.search(r"kTcThreads = 640;", CODE["baps_attention_tc.cuh"])
+    assert "kTcThreads = kTcSplit.threads;" in CODE["baps_attention_tc.cuh"]
+    assert re.search(r"kTcSplit = \{640, ", CODE["baps_register_split.cuh"])
 
 
 def test_no_load_asks_for_data_that_never_changes():
