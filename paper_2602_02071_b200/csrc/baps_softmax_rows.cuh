@@ -216,6 +216,14 @@ __device__ __forceinline__ void scan_groups(int ngroups, int bpg, int nb, float2
     if (lane == 0) *s_mfinal = m;
 }
 
+// Float output of whole power-of-two rows in 128-column blocks: these kernels run at the copy bandwidth, and what the
+// fewer instructions of the form above save them they lose in HBM.  With the weights moved to the final max in the second
+// pass (not together with the division in the third) and the block parameters handed round by shuffles, 2^27 / 2^28
+// logits take at 4K columns 167 / 337 us instead of 172 / 348, at 16K 176 / 351 instead of 178 / 359, at 32K 170 / 327
+// instead of 175 / 353.  64-column blocks, 8-bit output and other lengths lose 2 to 5 % by it (3200 columns 175 -> 180).
+template <int BK, bool CODES, bool FULL>
+constexpr bool kScaledEarly = !CODES && BK == 128 && FULL;
+
 // Largest maximum of a warp's vector (mx: the lane's block), kept by the lanes for the group's.
 template <int BPW>
 __device__ __forceinline__ float whole_warp_max(float mx)
@@ -356,19 +364,24 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
         const int jmine = chunk(lane / BPW) * BPW + lane % BPW;      // the block whose parameters I work out
         const unsigned slow = prepare_blocks<BPW, CODES>(s_blk, kNoGroup, jmine, lane < NV * BPW && (FULL || jmine < nb), lambda, s_mfinal,
                                                          CODES ? out.block_exp + row * nb : nullptr);
+        constexpr bool kEarly = kScaledEarly<BK, CODES, FULL>;
+        const float2 own = kEarly && lane < NV * BPW ? s_blk[jmine] : make_float2(0.f, 0.f);
         float dsum = 0.f;
         // ---- pass 2: weights against the block's own max (8-bit output: codes), their sum against the final max
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             if (!has(k)) break;
-            const float2 bp = s_blk[chunk(k) * BPW + lane / LPB];
+            const float2 bp = kEarly ? make_float2(__shfl_sync(0xffffffffu, own.x, k * BPW + lane / LPB),
+                                                   __shfl_sync(0xffffffffu, own.y, k * BPW + lane / LPB))
+                                     : s_blk[chunk(k) * BPW + lane / LPB];
             const bool any_pos = (slow >> (k * BPW)) & 1u;
             if constexpr (CODES) {
                 uint32_t *c4 = reinterpret_cast<uint32_t *>(out.codes + row * cols);
                 dsum = fmaf(emit_codes(c4 + chunk(k) * 32 + lane, table_words(v[k], bp.x, any_pos, rep, s_lut)), bp.y, dsum);
             } else {
                 v[k] = vector_weights(v[k], bp.x, any_pos, k == 0 && warp == 0 && lane < LPB, rep, s_lut);
-                dsum = fmaf(sum4(v[k]), bp.y, dsum);
+                if (kEarly) v[k] = make_float4(v[k].x * bp.y, v[k].y * bp.y, v[k].z * bp.y, v[k].w * bp.y);
+                dsum = kEarly ? dsum + sum4(v[k]) : fmaf(sum4(v[k]), bp.y, dsum);
             }
         }
         dsum = warp_sum(dsum);
@@ -386,7 +399,7 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
             float4 *p4 = reinterpret_cast<float4 *>(out.probs + row * cols);
 #pragma unroll
             for (int k = 0; k < NV; ++k)
-                if (has(k)) store_scaled(p4 + chunk(k) * 32 + lane, v[k], s_blk[chunk(k) * BPW + lane / LPB].y * dinv);
+                if (has(k)) store_scaled(p4 + chunk(k) * 32 + lane, v[k], kEarly ? dinv : s_blk[chunk(k) * BPW + lane / LPB].y * dinv);
         }
         // (no barrier here: what the next row writes first, s_blk[].x, was last read before the third barrier
         // above; s_blk[].y, s_mfinal and s_red are written behind the next row's first and second barrier,
@@ -632,19 +645,24 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
         const int jmine = warp * NV * BPW + lane;      // the block whose parameters I work out
         const unsigned slow = prepare_blocks<BPW, CODES>(s_blk, kNoGroup, jmine, lane < NV * BPW && (FULL || jmine < nb), lambda, s_mfinal[grp],
                                                          CODES ? out.block_exp + row * nb : nullptr);
+        constexpr bool kEarly = kScaledEarly<BK, CODES, FULL>;
+        const float2 own = kEarly && lane < NV * BPW ? s_blk[jmine] : make_float2(0.f, 0.f);
         float dsum = 0.f;
         // ---- weights against the block's own max (8-bit output: codes), their sum against the final max ----
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             if (!has(k)) break;
-            const float2 bp = s_blk[chunk(k) * BPW + lane / LPB];
+            const float2 bp = kEarly ? make_float2(__shfl_sync(0xffffffffu, own.x, k * BPW + lane / LPB),
+                                                   __shfl_sync(0xffffffffu, own.y, k * BPW + lane / LPB))
+                                     : s_blk[chunk(k) * BPW + lane / LPB];
             const bool any_pos = (slow >> (k * BPW)) & 1u;
             if constexpr (CODES) {
                 uint32_t *c4 = reinterpret_cast<uint32_t *>(out.codes + row * cols);
                 dsum = fmaf(emit_codes(c4 + chunk(k) * 32 + lane, table_words(v[k], bp.x, any_pos, rep, s_lut)), bp.y, dsum);
             } else {
                 v[k] = vector_weights(v[k], bp.x, any_pos, k == 0 && warp == 0 && lane < LPB, rep, s_lut);
-                dsum = fmaf(sum4(v[k]), bp.y, dsum);
+                if (kEarly) v[k] = make_float4(v[k].x * bp.y, v[k].y * bp.y, v[k].z * bp.y, v[k].w * bp.y);
+                dsum = kEarly ? dsum + sum4(v[k]) : fmaf(sum4(v[k]), bp.y, dsum);
             }
         }
         dsum = warp_sum(dsum);
@@ -665,7 +683,7 @@ softmax_rows_group_kernel(const float *__restrict__ logits, RowsOut out, int64_t
             float4 *p4 = reinterpret_cast<float4 *>(out.probs + row * cols);
 #pragma unroll
             for (int k = 0; k < NV; ++k)
-                if (has(k)) store_scaled(p4 + chunk(k) * 32 + lane, v[k], s_blk[chunk(k) * BPW + lane / LPB].y * dinv);
+                if (has(k)) store_scaled(p4 + chunk(k) * 32 + lane, v[k], kEarly ? dinv : s_blk[chunk(k) * BPW + lane / LPB].y * dinv);
         }
         // (no barrier here: what the next row writes first, s_blk[].x, was last read before the third barrier
         // above; s_blk[].y, s_mfinal and s_red are written behind the next row's first and second barrier,
@@ -773,7 +791,10 @@ softmax_rows_warp_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
 // Launch the variant for the row length (see the head of this file).
 // Grids: several times the CTAs that are resident at once (a few rows per CTA), so that the hardware
 // scheduler evens out the SMs; measured on 2^28 logits, a grid of exactly the resident CTAs -- each
-// with a fixed share of the rows -- loses 5 to 10 % to the slowest SM.
+// with a fixed share of the rows -- loses 5 to 10 % to the slowest SM.  CTAs per SM, measured on 2^27 / 2^28 logits,
+// float output: 4K columns 4 167 / 337 us, 6 170 / 332, 8 175 / 328 (64-column blocks: 4 168 / 332, 6 175 / 330);
+// 16K columns 2 187 / 367, 4 176 / 351, 8 173 / 340, 12 179 / 338; 8-bit output 2 107 / 202, 8 114 / 209 and, at
+// 4K columns, 4 115 / 215, 6 121 / 221.
 // Up to 8K columns the rows are register-resident and several rows share a CTA and its tables
 // (softmax_rows_group_kernel: 16 or 32 elements per thread); up to 1152 a warp per row needs no barrier at
 // all.  At 16K and 32K only one or two CTAs fit an SM, and the ring lets the next row's read overlap
@@ -812,9 +833,9 @@ inline baps_status softmax_rows_dispatch(const float *logits, const RowsOut &out
     case 1024:  return warp_rows(softmax_rows_warp_kernel<BK, 8, 1, CODES>, 1);
     case 1152:  return warp_rows(softmax_rows_warp_kernel<BK, 9, 1, CODES>, 1);
     case 2048:  return group(softmax_rows_group_kernel<BK, 128, 4, 4, CODES, true>, 128, 512, 16);
-    case 4096:  return group(softmax_rows_group_kernel<BK, 256, 4, 4, CODES, true, CODES>, 256, 1024, 4);
+    case 4096:  return group(softmax_rows_group_kernel<BK, 256, 4, 4, CODES, true, CODES>, 256, 1024, kScaledEarly<BK, CODES, true> ? 6 : 4);
     case 8192:  return group(softmax_rows_group_kernel<BK, 256, 8, 4, CODES, false>, 256, 1024, 4);
-    case 16384: return ring(softmax_rows_ring_kernel<BK, 512, CODES, CODES>, 512, 65536, 65536, 2);
+    case 16384: return ring(softmax_rows_ring_kernel<BK, 512, CODES, CODES>, 512, 65536, 65536, CODES ? 2 : 8);
     case 32768: return ring(softmax_rows_ring_kernel<BK, 1024, CODES>, 1024, 131072, 131072, 2);
     case 65536: return ring(softmax_rows_quarters_kernel<BK, CODES>, 1024, 196608, 196608, 2);
     }
