@@ -68,6 +68,9 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
     // ---- setup: the producer starts the first loads, the softmax warps fill their tables, then all meet
     const int n_early = 2 * J < L::kStages ? 2 * J : L::kStages;     // loads that need no free stage
     auto load_kv = [&](int l) {                                      // l = 2 j: K_j, 2 j + 1: V_j
+#ifdef BAPS_TEST_SKIP_LOAD
+        if (l == g_test_skip_load) return;                           // this tile never arrives
+#endif
         const int s = stage_of(l);
         mbar_arrive_expect_tx(bar(BKF + s), (uint32_t)L::kTileBytes);
         tma_load_2d(sbase + L::kKvOff + s * L::kTileBytes, (l & 1) ? &mv : &mk, 0, kv_row0 + (l >> 1) * 128, bar(BKF + s));

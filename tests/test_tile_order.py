@@ -1,55 +1,11 @@
 """The order in which the CTAs of the fused attention take query tiles and heads (``csrc/baps_tile_order.cuh``,
 compiled here as plain C++): every tile once, chunks of kv heads even, and the SMs as evenly busy as without chunks."""
-import ctypes
 import heapq
 import random
-import subprocess
 
 import pytest
 
-from paper_2602_02071_b200 import build
-
-SHIM = r"""
-#include "baps_tile_order.cuh"
-using namespace baps;
-extern "C" int one_tile(long long heads, int nq, int causal, int sms) { return one_tile_per_cta(heads, nq, causal, sms); }
-extern "C" void chunks(long long kv, long long bytes, long long per_kv, int causal, int sms, int per_sm, int *out)
-{ const KvChunks c = kv_chunks(kv, bytes, per_kv, causal, sms, per_sm); out[0] = c.size; out[1] = c.wide; }
-extern "C" void items(int H, int Hkv, int npairs, int size, int wide, int n, int *out)
-{
-    const KvChunks c = {size, wide};
-    for (int i = 0; i < n; ++i) {
-        const WorkItem w = work_item(H, Hkv, npairs, c, i);
-        out[4 * i] = w.tile; out[4 * i + 1] = w.h; out[4 * i + 2] = w.hk; out[4 * i + 3] = w.b;
-    }
-}
-"""
-SMS = 148
-
-
-@pytest.fixture(scope="module")
-def order(tmp_path_factory):
-    d = tmp_path_factory.mktemp("order")
-    (d / "shim.cpp").write_text(SHIM)
-    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", build.CSRC, "-o", str(d / "shim.so"),
-                    str(d / "shim.cpp")], check=True)
-    lib = ctypes.CDLL(str(d / "shim.so"))
-    ll, i = ctypes.c_longlong, ctypes.c_int
-    lib.one_tile.argtypes = [ll, i, i, i]
-    lib.chunks.argtypes = [ll, ll, ll, i, i, i, ctypes.POINTER(i)]
-    lib.items.argtypes = [i, i, i, i, i, i, ctypes.POINTER(i)]
-
-    def tiles(B, H, Hkv, npairs, kv_bytes, causal, per_sm, whole=False):
-        c = (ctypes.c_int * 2)(B * Hkv, 0)
-        if not whole:
-            lib.chunks(B * Hkv, kv_bytes, npairs * (H // Hkv), causal, SMS, per_sm, c)
-        n = B * H * npairs
-        out = (ctypes.c_int * (4 * n))()
-        lib.items(H, Hkv, npairs, c[0], c[1], n, out)
-        return (c[0], c[1]), [tuple(out[4 * k:4 * k + 4]) for k in range(n)]
-
-    tiles.one = lambda heads, nq, causal: bool(lib.one_tile(heads, nq, causal, SMS))
-    return tiles
+from tile_order import SMS, one_tile_per_cta, tiles
 
 
 def makespan(items, nq, pairs, slots):
@@ -72,31 +28,31 @@ SHAPES = [(2, 32, 8, 8192, 384), (4, 32, 8, 4096, 384), (1, 36, 9, 8192, 512), (
           (23, 7, 7, 1024, 256), (9, 15, 5, 2048, 512), (301, 2, 1, 1024, 512), (1, 1, 1, 128, 512), (3, 6, 2, 640, 256)]
 
 
-def check(order, B, H, Hkv, S, key_bytes):
+def check(B, H, Hkv, S, key_bytes):
     nq = S // 128
-    pairs = key_bytes != 256 and not order.one(B * H, nq, True)
+    pairs = key_bytes != 256 and not one_tile_per_cta(B * H, nq, True)
     per_sm = 2 if key_bytes == 256 else 1
     n = (nq + 1) // 2 if pairs else nq
     for causal in (True, False):
-        (size, wide), items = order(B, H, Hkv, n, S * key_bytes, causal, per_sm)
+        (size, wide), items = tiles(B, H, Hkv, n, S * key_bytes, causal, per_sm)
         assert sorted((b, h, t) for t, h, _, b in items) == [(b, h, t) for b in range(B) for h in range(H) for t in range(n)]
         assert all(hk == h // (H // Hkv) for _, h, hk, _ in items)
         assert 0 <= wide <= B * Hkv and (B * Hkv - wide * (size + 1)) % size == 0      # all of one size but for one head
-    _, chunked = order(B, H, Hkv, n, S * key_bytes, True, per_sm)
-    _, whole = order(B, H, Hkv, n, S * key_bytes, True, per_sm, whole=True)
+    _, chunked = tiles(B, H, Hkv, n, S * key_bytes, True, per_sm)
+    _, whole = tiles(B, H, Hkv, n, S * key_bytes, True, per_sm, whole=True)
     # 3 %: what reading K and V from L2 gives at these sizes; a ragged last chunk costs 5 to 35 % in this estimate
     assert makespan(chunked, nq, pairs, per_sm * SMS) <= 1.03 * makespan(whole, nq, pairs, per_sm * SMS)
 
 
 @pytest.mark.parametrize("B,H,Hkv,S,key_bytes", SHAPES)
-def test_every_tile_once_in_even_chunks_that_keep_the_sms_busy(order, B, H, Hkv, S, key_bytes):
-    check(order, B, H, Hkv, S, key_bytes)
+def test_every_tile_once_in_even_chunks_that_keep_the_sms_busy(B, H, Hkv, S, key_bytes):
+    check(B, H, Hkv, S, key_bytes)
 
 
-def test_random_shapes(order):
+def test_random_shapes():
     rng = random.Random(5)
     for _ in range(60):
         Hkv, g, B = rng.randint(1, 48), rng.choice([1, 1, 2, 3, 4, 8]), rng.choice([1, 1, 2, 3, 5])
         nq, key_bytes = rng.choice([1, 3, 8, 16, 31, 64]), rng.choice([256, 384, 512])
         if B * Hkv * g * nq <= 30000:
-            check(order, B, Hkv * g, Hkv, 128 * nq, key_bytes)
+            check(B, Hkv * g, Hkv, 128 * nq, key_bytes)
