@@ -11,6 +11,7 @@ import torch
 import oracle
 from paper_2602_02071_b200 import binding, workloads
 from parity import EPS_REL, gate_attention
+from tile_order import form
 
 pytestmark = pytest.mark.gpu
 
@@ -246,13 +247,13 @@ def test_restart_rates_rejects_small_scratch():
 
 
 @pytest.mark.parametrize("causal", [False, True])
-@pytest.mark.parametrize("D", [64, 128])
-@pytest.mark.parametrize("S", [128, 384, 512])
+@pytest.mark.parametrize("S,D", [(256, 128), (384, 128), (512, 128), (128, 64), (384, 64), (512, 64)])
 def test_one_and_two_query_tiles_per_cta_agree(S, D, causal):
     """A few heads (one query tile per CTA) and the same heads repeated until the SMs are full several times
     over (two tiles per CTA, an odd one left over at S = 384; D = 64: the kernel with two CTAs per SM): the same
     decisions, max and restarts, the same bits but for the order of the row sum at D = 64 (128 addends per tile
     and thread at most: 2^-17), which may move a bf16 output by one unit."""
+    assert form(D, 6, S // 128, causal) == "one tile" and form(D, 6 * 256, S // 128, causal) != "one tile"
     g = torch.Generator(device="cuda"); g.manual_seed(S + D)
     q, k, v = (torch.randn(1, h, S, D, device="cuda", generator=g).bfloat16() for h in (6, 2, 2))
     few = binding.baps_attention_fwd_ex(q, k, v, causal=causal, block_q=128, block_k=128)
@@ -281,15 +282,60 @@ def test_two_ctas_per_sm_d64_against_the_checker(causal, lam):
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("B,Hkv,g,D", [(23, 7, 1, 64), (9, 5, 3, 128), (301, 1, 2, 128)])
 def test_chunks_of_heads_cover_every_tile(B, Hkv, g, D, causal):
-    """Head counts that leave the last chunk of kv heads ragged: every (batch, head) as when run alone."""
-    S = 2048 if D == 128 and B < 100 else 1024
+    """Head counts that the chunks of kv heads do not divide: a few different heads in no regular order, and every
+    (batch, head) of the result as that head gives when run alone."""
+    S, n = 2048 if D == 128 and B < 100 else 1024, 5
     gen = torch.Generator(device="cuda"); gen.manual_seed(B)
-    q, k, v = (torch.randn(B, h, S, D, device="cuda", generator=gen).bfloat16() for h in (Hkv * g, Hkv, Hkv))
+    pool = [torch.randn(n, h, S, D, device="cuda", generator=gen).bfloat16() for h in (g, 1, 1)]
+    pick = torch.randint(0, n, (B * Hkv,), device="cuda", generator=gen)
+    q, k, v = (t[pick].reshape(B, Hkv * t.shape[1], S, D) for t in pool)
     out = torch.full_like(q, float("nan"))
     binding.baps_attention_fwd(q, k, v, causal=causal, out=out)
-    assert not torch.isnan(out).any()
-    for b, h in ((0, 0), (B // 2, Hkv - 1), (B - 1, 0), (B - 1, Hkv - 1)):
-        alone = binding.baps_attention_fwd(q[b:b + 1, h * g:(h + 1) * g].contiguous(), k[b:b + 1, h:h + 1].contiguous(),
-                                           v[b:b + 1, h:h + 1].contiguous(), causal=causal)
-        # (D = 64: the lone head takes the other kernel, whose row sum is added up in another order)
-        assert torch.allclose(out[b, h * g:(h + 1) * g].float(), alone[0].float(), rtol=2.0 ** -7, atol=0)
+    alone = torch.cat([binding.baps_attention_fwd(*(t[i:i + 1] for t in pool), causal=causal) for i in range(n)])
+    want = alone[pick].reshape(out.shape)
+    if D == 128:
+        assert torch.equal(out, want)
+    else:       # the lone head takes the other kernel, whose row sum is added up in another order
+        assert torch.allclose(out.float(), want.float(), rtol=2.0 ** -7, atol=0)
+
+
+def _check_repeated(w, n, want_form, lam=1, qkv=None, max_near_frac=0.01):
+    """The heads of one small problem repeated n times, a grid that takes `want_form`: one copy against the checker,
+    and all copies alike."""
+    nq = w.S // 128
+    assert form(w.D, w.H * n, nq, w.causal) == want_form
+    q, k, v = qkv or workloads.make_qkv(w)
+    st = _run_gpu(w, *(t.cuda().repeat(n, 1, 1, 1) for t in (q, k, v)), lam=lam)
+    for t in (st.out, st.out_f32, st.row_m, st.row_d, st.restarts):
+        assert torch.equal(t, t[:1].expand_as(t))
+    ref = oracle.attention(_np(q), _np(k), _np(v), causal=w.causal, block_q=128, block_k=128, lam=lam)
+    gate_attention(st.out_f32[n // 2].cpu().numpy(), ref, what=f"{want_form} S={w.S} causal={w.causal} lam={lam}",
+                   max_near_frac=max_near_frac)
+    clear = ref.row_margin >= EPS_REL
+    assert np.array_equal(st.row_m[0].cpu().numpy().reshape(ref.row_m.shape)[clear], ref.row_m[clear])
+    got = st.restarts[0].cpu().numpy().reshape(-1)
+    assert np.array_equal(got[clear.all(axis=1)], ref.restarts.reshape(-1)[clear.all(axis=1)])
+    return st, ref
+
+
+@pytest.mark.parametrize("S,causal,lam", [(768, True, 0), (640, True, 1), (768, True, 2), (896, False, 3), (256, False, 1)])
+def test_two_query_tiles_per_cta_against_the_checker(S, causal, lam):
+    """Outlier keys (restarts), positive T, even and odd numbers of query tiles, every lambda."""
+    w = workloads.AttnWorkload("t", 1, 4, 2, S, 128, causal, 128, 128, outlier_frac=0.01, seed=300 + S + lam)
+    st, _ = _check_repeated(w, 160, "two tiles", lam=lam)
+    assert int(st.restarts.sum()) > 0 or S == 256
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("D,want_form", [(128, "two tiles"), (64, "two CTAs per SM")])
+def test_rising_max_rebases_the_output(D, want_form, causal):
+    """The row maximum rises by more than five with every key tile, past the exponent of 64 at which O~ and d are
+    rebased (its last value against its first is asserted), on grids that take the forms of the long prefills."""
+    S, H = 2048, 2
+    w = workloads.AttnWorkload("rising", 1, H, H, S, D, causal, 128, 128)
+    qkv = workloads.make_rising_max_qkv(S, H=H, D=D, rise_per_tile=5.2)
+    # (every row takes 15 decisions here, each with a rounding boundary of its own)
+    st, _ = _check_repeated(w, 64, want_form, qkv=qkv, max_near_frac=0.10)
+    q, k = qkv[0].float(), qkv[1].float()
+    first = (q[:, :, -128:] @ k[:, :, :128].transpose(-1, -2)).amax(-1) * 1.4426950408889634 / D ** 0.5
+    assert float((st.row_m[0, :, -128:].cpu() - first[0]).min()) > 66
