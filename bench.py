@@ -43,17 +43,17 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # None where no capture of that workload exists.
 NCU_CAPTURES = {
     # profiles/attention_tc_kernel_c5_long_context_dram.txt: one launch of the full workload
-    # (1915.3 MB read + 249.7 MB written, 43.9 % of cycles)
-    "c5_long_context": {"traffic": 2165.0e6, "tensor_pipe_active_pct": 43.9},
-    # profiles/attention_tc_kernel_c2_llm_prefill_mha.txt: 146.5 MB read + 14.5 MB written
-    "c2_llm_prefill_mha": {"traffic": 161.0e6, "tensor_pipe_active_pct": 37.7},
+    # (404.1 MB read + 239.3 MB written, 44.0 % of cycles)
+    "c5_long_context": {"traffic": 643.4e6, "tensor_pipe_active_pct": 44.0},
+    # profiles/attention_tc_kernel_c2_llm_prefill_mha.txt: 145.2 MB read + 14.3 MB written
+    "c2_llm_prefill_mha": {"traffic": 159.6e6, "tensor_pipe_active_pct": 37.6},
 }
 
-# Thread instructions per score element of the fused kernel, from smsp__inst_executed.sum of the committed
-# captures (profiles/attention_tc_kernel_long_causal_s16384.txt: 415.7 M warp instructions for 1.08e9
-# scores; profiles/attention_tc_kernel_d64_vit_b8_s1024.txt: 54.2 M for 1.34e8), and the issue peak of the
-# part: 148 SMs x 4 schedulers x 32 lanes per clock.
-INSTR_PER_SCORE = {128: 12.3, 64: 12.9}
+# Thread instructions per score element of the fused kernels, from smsp__inst_executed.sum of the committed
+# captures (profiles/attention_tc_kernel_long_causal_s16384.txt: 12.18; configuration 2 with its outlier keys 12.41;
+# profiles/attention_d64_kernel_vit_b8_s1024.txt: 12.04), and the issue peak of the part: 148 SMs x 4 schedulers x
+# 32 lanes per clock.
+INSTR_PER_SCORE = {128: 12.2, 64: 12.0}
 ISSUE_LANES_PER_CLOCK = 148 * 4 * 32
 
 
@@ -450,6 +450,8 @@ PROFILE_CASES = {
     "attn_c3": workloads.WORKLOADS["c3_llm_prefill_gqa"],
     "attn_c4": workloads.WORKLOADS["c4_vit_encoder"],
     "attn_c5": workloads.WORKLOADS["c5_long_context"],
+    "attn_one_tile": workloads.AttnWorkload("profile_attn_one_tile", 1, 8, 8, 4096, 128, True, 128, 128),
+    "attn_fp8": workloads.AttnWorkload("profile_attn_fp8", 1, 8, 2, 16384, 128, True, 128, 128),      # 8-bit Q / K
     "attn_d64": workloads.AttnWorkload("profile_attn_d64", 8, 16, 16, 1024, 64, False, 128, 128, key_bias_var=0.5),
 }
 
@@ -465,6 +467,9 @@ def run_profile_case(name: str, launches: int = 3, warmup: int = 3):
         q, k, v = workloads.make_qkv(w, device="cuda")
         out = torch.empty_like(q)
         fn = lambda: binding.baps_attention_fwd(q, k, v, causal=w.causal, out=out)
+        if name == "attn_fp8":
+            (q8, qs, _), (k8, ks, _) = (workloads.quantize_e4m3_tiles(t) for t in (q, k))
+            fn = lambda: binding.baps_attention_fwd_fp8(q8, k8, v, qs, ks, causal=w.causal, want_stats=False, out=out)
         work, unit = w.flops / 1e12, "TFLOP/s"
     elif name in ("encode", "decode", "exp2_map") or name.startswith("softmax_rows_"):   # softmax_rows[_codes]_<cols>
         n = 1 << 27                                      # 512 MB of fp32: larger than L2
@@ -482,12 +487,12 @@ def run_profile_case(name: str, launches: int = 3, warmup: int = 3):
             fn, work = (lambda: binding.baps_exp2_hif8(codes, codes2)), 2.0 * n / 1e9
         elif name.startswith("softmax_rows_codes_"):
             cols = int(name.rsplit("_", 1)[1])
-            xr = x.view(n // cols, cols)
-            fn, work = (lambda: binding.baps_softmax_rows_codes(xr, 128)), 5.0 * n / 1e9
+            xr = x[:n // cols * cols].view(-1, cols)
+            fn, work = (lambda: binding.baps_softmax_rows_codes(xr, 128)), 5.0 * xr.numel() / 1e9
         else:
             cols = int(name.rsplit("_", 1)[1])
-            xr, yr = x.view(n // cols, cols), y.view(n // cols, cols)
-            fn, work = (lambda: binding.baps_softmax_rows(xr, 128, yr)), 8.0 * n / 1e9
+            xr, yr = x[:n // cols * cols].view(-1, cols), y[:n // cols * cols].view(-1, cols)
+            fn, work = (lambda: binding.baps_softmax_rows(xr, 128, yr)), 8.0 * xr.numel() / 1e9
         unit = "GB/s"
     else:
         raise SystemExit(f"unknown profile case {name}")
@@ -585,7 +590,7 @@ def main():
         "tensor_pipe_active_pct_ncu": cap.get("tensor_pipe_active_pct"),
         "traffic": cap.get("traffic"),
         "algorithmic_bytes": float(2 * (2 * w.B * w.H + 2 * w.B * w.Hkv) * w.S * w.D),
-        "kernel": "attention_tc_kernel<%d, false>" % w.D, "best_ms": float(np.min(times)),
+        "kernel": "attention_d64_kernel" if w.D == 64 else "attention_tc_kernel<128, Algorithm 1>", "best_ms": float(np.min(times)),
         "median_ms": float(np.median(times)),
         "ms_x_sm_mhz": kernel_ms * clocks["sm_mhz"] if clocks["sm_mhz"] else None,
         "issue_roofline": issue_roofline(w, kernel_ms, clocks["sm_mhz"]),

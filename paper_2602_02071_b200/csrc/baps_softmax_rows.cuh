@@ -415,7 +415,7 @@ softmax_rows_ring_kernel(const float *__restrict__ logits, RowsOut out, int64_t 
 // four significant bits; block 0, in high precision, is formed again from its logits), so that the
 // pieces of quarters 2 and 3 take the next row before the output is written.  The transit piece takes quarter 1
 // once quarter 0 sits in registers and the next row's quarter 0 once quarter 1 does -- so of the next row only
-// quarter 1 is waited for in the open.  Five barriers per row.
+// quarter 1 is waited for in the open.  Four barriers per row.
 template <int BK, bool CODES, bool FULL = true>
 __global__ void __launch_bounds__(1024, 1)
 softmax_rows_quarters_kernel(const float *__restrict__ logits, RowsOut out, int64_t rows, int lambda, int cols_)
