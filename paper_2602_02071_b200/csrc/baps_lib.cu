@@ -33,10 +33,11 @@ baps_status attention_f32_launch(const AttnF32Params &p, cudaStream_t st)
 {
     using L = AfLayout<BLK>;
     // the limit is state of the kernel, which other threads may be launching with other head sizes: never anything but
-    // the largest head's (not set at all where the default does: 0.4 us of an 8.5 us call)
+    // the largest head's (not set at all where the default of 48 KB holds this and the kernel's static arrays, 1.4 KB:
+    // 0.4 us of an 8.5 us call)
     const size_t smem = sizeof(float) * (size_t)L(p.D).total;
     const int most = (int)sizeof(float) * L(128).total;
-    if (smem > 48 * 1024 &&
+    if (smem + 2048 > 48 * 1024 &&
         cudaFuncSetAttribute(attention_f32_kernel<BLK>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
         return BAPS_ERR_CUDA;
     const dim3 grid((unsigned)(p.S / BLK) * kAfCluster, p.H, p.B);

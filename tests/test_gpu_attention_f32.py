@@ -1,4 +1,8 @@
-"""GPU parity: the CUDA-core float32 attention kernel against the CPU checker."""
+"""GPU parity: the float32 attention kernel (double-precision scores) against the CPU checker."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -92,3 +96,25 @@ def test_f32_kernel_head_sizes(D, bq, S):
     v[:, :, -1] = float("inf")                  # only the last query sees the last key
     out = binding.baps_attention_fwd_f32(q, k, v, causal=True, block_q=bq, block_k=bq)
     assert torch.equal(out[:, :, :-1], st.out_f32[:, :, :-1])
+
+
+_ALL_HEAD_SIZES = """
+import sys; sys.path[:0] = {path!r}
+import torch
+from paper_2602_02071_b200 import binding
+torch.manual_seed(3)
+for D in range(4, 129, 4):                      # ascending: no call finds a limit that a larger head has raised
+    for block in (64, 128):
+        q, k, v = (torch.randn(1, 1, 128, D, device="cuda") for _ in range(3))
+        out = binding.baps_attention_fwd_ex(q, k, v, causal=False, block_q=block, block_k=block, mode=binding.MODE_EXACT).out
+        want = torch.softmax(q.double() @ k.double().mT / D ** 0.5, -1) @ v.double()
+        err = float((out - want).abs().max())
+        assert err < 1e-4, (D, block, err)      # 128 products and exponentials in float32
+"""
+
+
+def test_every_head_size_in_a_fresh_process():
+    """Head sizes whose shared memory, with the kernel's own arrays, just passes the default limit of 48 KB."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", _ALL_HEAD_SIZES.format(path=[root])], capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr[-2000:]
