@@ -143,7 +143,7 @@ typedef struct {
 } baps_stats;
 
 /* dtype: BAPS_DTYPE_BF16 selects the tensor-core kernel (same supported set as
- * baps_attention_fwd), BAPS_DTYPE_F32 the CUDA-core kernel.  `out` may be NULL if
+ * baps_attention_fwd), BAPS_DTYPE_F32 the float32 kernel.  `out` may be NULL if
  * stats->out_f32 is given.  opts == NULL means {1, BAPS_MODE_E2E_HIF8, 0, 0}.               */
 baps_status baps_attention_fwd_ex(const void *q, const void *k, const void *v, void *out,
                                   int B, int H, int Hkv, int S, int D, int causal,

@@ -98,7 +98,7 @@ def test_key_bias_non_causal_d64():
 
 
 def test_matches_cuda_core_kernel_and_plain_entry_point():
-    """Same inputs through the CUDA-core fp32 kernel (double-precision scores) and through the
+    """Same inputs through the float32 kernel (double-precision scores) and through the
     plain bf16 entry point."""
     w = workloads.AttnWorkload("t", 1, 2, 1, 512, 128, True, 128, 128, seed=8)
     q, k, v = workloads.make_qkv(w, device="cuda")
@@ -300,7 +300,7 @@ def test_chunks_of_heads_cover_every_tile(B, Hkv, g, D, causal):
 
 
 def _check_repeated(w, n, want_form, lam=1, qkv=None, max_near_frac=0.01):
-    """The heads of one small problem repeated n times, a grid that takes `want_form`: one copy against the checker,
+    """The heads of one small problem repeated n times, a grid that takes `want_form`: one copy against the oracle,
     and all copies alike."""
     nq = w.S // 128
     assert form(w.D, w.H * n, nq, w.causal) == want_form
@@ -319,7 +319,7 @@ def _check_repeated(w, n, want_form, lam=1, qkv=None, max_near_frac=0.01):
 
 
 @pytest.mark.parametrize("S,causal,lam", [(768, True, 0), (640, True, 1), (768, True, 2), (896, False, 3), (256, False, 1)])
-def test_two_query_tiles_per_cta_against_the_checker(S, causal, lam):
+def test_two_query_tiles_per_cta_against_the_oracle(S, causal, lam):
     """Outlier keys (restarts), positive T, even and odd numbers of query tiles, every lambda."""
     w = workloads.AttnWorkload("t", 1, 4, 2, S, 128, causal, 128, 128, outlier_frac=0.01, seed=300 + S + lam)
     st, _ = _check_repeated(w, 160, "two tiles", lam=lam)
