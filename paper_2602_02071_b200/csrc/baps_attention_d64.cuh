@@ -101,15 +101,7 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
         allow_next_kernel();
         if (lane == 0) { tma_prefetch_desc(&mq); tma_prefetch_desc(&mk); tma_prefetch_desc(&mv); }
     } else if (warp < kD64SoftmaxWarps) {
-        float4 *rep = reinterpret_cast<float4 *>(smem + L::kLutRepOff);
-        for (int e = tid; e < kLutRepEntries; e += kD64SoftmaxWarps * 32) {
-            const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
-            const float4 w4 = make_float4(w, w, w, w);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) rep[e * 8 + i] = w4;
-        }
-        float *full = reinterpret_cast<float *>(smem + L::kLutFullOff);
-        for (int i = tid; i < kLutN; i += kD64SoftmaxWarps * 32) full[i] = g_w0.v[i];
+        fill_attention_tables(smem + L::kLutRepOff, smem + L::kLutFullOff, tid, kD64SoftmaxWarps * 32);
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -198,13 +190,12 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
         const uint32_t xrow = sbase + L::kXchgOff + (uint32_t)row * 8u;   // + 1024 * (j & 1); my slot + 4 ch
         const float c = p.c;
         const bool count_restarts = p.restarts != nullptr && warp == 0;
-        const float over_thr = p.lambda == 0 ? 1.1920928955078125e-07f
-                                             : (float)p.lambda + (p.lambda == 1 ? 0.0625f : 0.125f);
-        // m, m_ref and d as in attention_tc_kernel; d is the partial sum of my columns
-        float m = -INFINITY, m_ref = 0.f, d = 0.f;
+        const float over_thr = restart_threshold(p.lambda);
+        RowState st{-INFINITY, 0.f, 0.f, 0u};
         int n_restart = 0;
 
-        for (int j = 0; j < J; ++j) {
+        auto tile = [&](auto first, const int j) {
+            constexpr bool hp = decltype(first)::value;          // B0: the high-precision tile
             const uint32_t x_addr = xrow + (uint32_t)(j & 1) * 1024u;
             const bool diag = p.causal && j == qi;
             uint32_t r[32];
@@ -228,76 +219,46 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
             for (int i = 0; i < 4; ++i) g[4 + i] = max8(&r[8 * i]);
             const float hm = max3(max3(g[0], g[1], g[2]), max3(g[3], g[4], g[5]), fmaxf(g[6], g[7]));
             sts_f32(x_addr + 4u * (uint32_t)ch, hm);
-            const bool hp = j == 0;
             bool restart_tile = false;
-            if (!hp) {
-                restart_tile = named_bar_or(1, kD64SoftmaxWarps * 32, fmaf(hm, c, -m) >= over_thr);
-                if (count_restarts && restart_tile) ++n_restart;
+            if constexpr (hp) named_bar_sync(2 + q4, 64);
+            else restart_tile = named_bar_or(1, kD64SoftmaxWarps * 32, fmaf(hm, c, -st.m) >= over_thr);
+            const float2 pm = lds_f32x2(x_addr);
+            const float mx = fmaxf(pm.x, pm.y);
+            // ---- decisions (Algorithm 1) -------------------------------------------------------------------
+            bool changed = false;                 // the max moves in some row of the warp (with or without a restart)
+            float m_next = st.m;
+            if constexpr (hp) {
+                st.m = st.m_ref = m_next = int_max(mx, c);
             } else {
-                named_bar_sync(2 + q4, 64);
-            }
-            float mx;
-            {
-                float m0, m1;
-                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m0), "=f"(m1) : "r"(x_addr) : "memory");
-                mx = fmaxf(m0, m1);
-            }
-            // ---- decisions (Algorithm 1), as in attention_tc_kernel ---------------------------------------
-            const float um = hp ? -1.f : fmaf(mx, c, -m);
-            const bool any_posf = __any_sync(0xffffffffu, um > 0.f);
-            float m_new, mref_w;
-            if (hp || restart_tile) {
-                float smax = ceilf(mx * c);
-                if (fmaf(mx, c, -smax) > 0.f) smax += 1.f;
-                m_new = fmaxf(m, smax);
-                if (hp) m_ref = m_new;
-                mref_w = m_new;
-            } else {
-                m_new = m + ((um >= 1.1920928955078125e-07f ? 1.f : 0.f) + (um >= 1.0625f ? 1.f : 0.f) +
-                             (um >= 2.125f ? 1.f : 0.f));
-                mref_w = m;
-            }
-            {
-                const float kk = mref_w - m_ref;
-                const bool need = !hp && kk > 64.f;
-                if (__any_sync(0xffffffffu, need)) {
-                    const float f = need ? pow2_int(-kk) : 1.f;
-                    mbar_wait(bar(BD), (uint32_t)((j - 1) & 1), s_abort, &g_async_status, 0x330);
-                    tc_fence_after_sync();
-#pragma unroll 1
-                    for (int i0 = 0; i0 < 32; i0 += 16) {
-                        uint32_t o[16];
-                        tmem_ld16(o_addr + i0, o);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-                        tmem_st16(o_addr + i0, o);
-                    }
-                    d *= f;
-                    if (need) m_ref = mref_w;
+                const float um = fmaf(mx, c, -st.m);
+                changed = restart_tile || __any_sync(0xffffffffu, um > 0.f);
+                if (changed) {
+                    if (count_restarts && restart_tile) ++n_restart;
+                    m_next = st.decide(mx, c, um, restart_tile, [&](float f) {
+                        mbar_wait(bar(BD), (uint32_t)((j - 1) & 1), s_abort, &g_async_status, 0x330);
+                        tc_fence_after_sync();
+                        rescale_columns(o_addr, 32, f);
+                    });
                 }
             }
-            const int e_i = (int)(mref_w - m_ref);        // 0 .. 64; 0 in the first tile
-            const uint32_t escale = (uint32_t)e_i * 0x00800080u;
-            const bool pos_tile = !hp && !restart_tile && any_posf;
             // ---- weights -> bf16 P; row sum ---------------------------------------------------------------
             float sum = 0.f;
             uint64_t s01 = 0ull, s23 = 0ull;
-            const float mnv = mref_w * 7.52316384526264e-37f, cnv = -c * 7.52316384526264e-37f;     // 2^-120
+            const float mnv = st.m * 7.52316384526264e-37f, cnv = -c * 7.52316384526264e-37f;     // 2^-120
             const uint64_t cn2 = pack2(cnv, cnv), mn2 = pack2(mnv, mnv);
             auto weights = [&](int cc) {
                 uint32_t pk[16];
-                if (hp) {
-                    sum += hp16(&r[0], &pk[0], c, mref_w) + hp16(&r[16], &pk[8], c, mref_w);
+                if constexpr (hp) {
+                    sum += hp16(&r[0], &pk[0], c, st.m) + hp16(&r[16], &pk[8], c, st.m);
                 } else {
-                    fast16<false>(&r[0], &pk[0], cn2, mn2, escale, tb, s01, s23);
-                    fast16<false>(&r[16], &pk[8], cn2, mn2, escale, tb, s01, s23);
-                    if (pos_tile) {
+                    fast16<false>(&r[0], &pk[0], cn2, mn2, st.escale, tb, s01, s23);
+                    fast16<false>(&r[16], &pk[8], cn2, mn2, st.escale, tb, s01, s23);
+                    if (changed && !restart_tile) {
 #pragma unroll
                         for (int gg = 0; gg < 4; ++gg) {
-                            const bool gpos = fmaf(cc ? g[4 + gg] : g[gg], c, -mref_w) > 0.f;
+                            const bool gpos = fmaf(cc ? g[4 + gg] : g[gg], c, -st.m) > 0.f;
                             if (__any_sync(0xffffffffu, gpos))
-                                sum += fix8(&r[gg * 8], &pk[gg * 4], c, mref_w, escale, lut_full);
+                                sum += fix8(&r[gg * 8], &pk[gg * 4], c, st.m, st.escale, lut_full);
                             __syncwarp();
                         }
                     }
@@ -305,7 +266,7 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
                 tmem_st16(p_addr + cc * 16, pk);
             };
             // P V of the tile before has read its weights (long done, as a rule)
-            if (j > 0) {
+            if constexpr (!hp) {
                 mbar_wait(bar(BD), (uint32_t)((j - 1) & 1), s_abort, &g_async_status, 0x331);
                 tc_fence_after_sync();
             }
@@ -319,12 +280,16 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(BP));          // P is in place
-            float a0, a1, a2, a3;
-            unpack2(s01, a0, a1); unpack2(s23, a2, a3);
-            sum += (a0 + a1) + (a2 + a3);
-            d += sum * __int_as_float((127 + e_i) << 23);
-            m = m_new;
-        }
+            if constexpr (!hp) {
+                float a0, a1, a2, a3;
+                unpack2(s01, a0, a1); unpack2(s23, a2, a3);
+                sum += (a0 + a1) + (a2 + a3);
+            }
+            st.add(sum);
+            if (changed) st.move(m_next);
+        };
+        tile(std::true_type{}, 0);
+        for (int j = 1; j < J; ++j) tile(std::false_type{}, j);
         const bool ok = (*s_abort == 0);
 
         // ---- epilogue: O = O~ / d (each thread: its half of the output columns) -------------------------
@@ -332,11 +297,10 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
         tc_fence_after_sync();
         // the exchange buffer not used by the tile before (that one may still be read by the partner)
         const uint32_t x_addr = xrow + (uint32_t)(J & 1) * 1024u;
-        sts_f32(x_addr + 4u * (uint32_t)ch, d);
+        sts_f32(x_addr + 4u * (uint32_t)ch, st.d);
         named_bar_sync(2 + q4, 64);
-        float d0, d1;
-        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(d0), "=f"(d1) : "r"(x_addr) : "memory");
-        const float dtot = d0 + d1, dinv = 1.f / dtot;
+        const float2 pd = lds_f32x2(x_addr);
+        const float dtot = pd.x + pd.y, dinv = 1.f / dtot;
         const size_t grow = (size_t)q_row0 + row;                    // row in [B*H*S]
         // staged through the (now idle) Q tile, 16-byte chunks of a row XOR-swizzled with the row number, so
         // that the global stores are whole rows
@@ -376,8 +340,8 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
         }
         if (good) {
             if (ch == 0) {
-                if (p.row_m) p.row_m[grow] = m;
-                if (p.row_d) p.row_d[grow] = dtot * pow2_int(m_ref - m);
+                if (p.row_m) p.row_m[grow] = st.m;
+                if (p.row_d) p.row_d[grow] = dtot * pow2_int(st.m_ref - st.m);
             }
             if (count_restarts && lane == 0) p.restarts[(size_t)(b * p.H + h) * p.nq + qi] = n_restart;
         }

@@ -108,6 +108,24 @@ __device__ __forceinline__ float max3(float a, float b, float c)
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
+// upper halves of two words as one: a's in the low half, b's in the high
+__device__ __forceinline__ uint32_t upper_halves(float a, float b)
+{
+    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+// low half of a * byte 0 of b + high half of a * byte 1 of b + c
+__device__ __forceinline__ uint32_t dot_u16x2(uint32_t a, uint32_t b, uint32_t c)
+{
+    uint32_t d;
+    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
 // Hardware (named) barriers among the softmax warps: id 0 is __syncthreads.
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t nthreads)
 {
@@ -131,6 +149,12 @@ __device__ __forceinline__ float4 lds_f32x4(uint32_t addr)
 {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 lds_f32x2(uint32_t addr)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ void sts_u32x4(uint32_t addr, uint4 v)
@@ -161,7 +185,11 @@ __device__ __forceinline__ float pow2_int(float k)
 //         |T| < 2^-6 (weight 1), otherwise a normal number with biased exponent >= 1
 //   key = min(bits(x) >> 19, 192): exponent and top four mantissa bits (what HiF8 rounding with
 //         ties to the larger magnitude depends on); 192 stands for |T| >= 32 (weight 0) and is
-//         also where a positive T lands (sign bit set) -- those entries are redone by the caller
+//         also where a positive T lands (sign bit set) -- those entries are redone by the caller.
+//         Two keys are cut out, limited and masked at once, as the halves of one word, each eight times
+//         the key; the address of an entry's copy is then half * 16 + the lane's offset, one dot product
+//         instruction.  (Shift, minimum and multiply-add per element took 749 cycles per 128 x 128 tile
+//         with the rest of the weights and all warps busy; this form 676.)
 //   w   = table[key], 32 copies per entry, one per bank: no conflicts
 // The weights are exactly representable in bf16; the power-of-two factor 2^e (e >= 0) that
 // expresses them against the accumulators' reference max is added to the packed exponents.
@@ -183,8 +211,9 @@ __device__ __forceinline__ void fast16(const uint32_t *r, uint32_t *pk, uint64_t
         } else {
             unpack2(fma2_ftz(pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), cn2, mn2), x0, x1);
         }
-        a[i] = min(__float_as_uint(x0) >> 19, 192u) * 128u + tb;
-        a[i + 1] = min(__float_as_uint(x1) >> 19, 192u) * 128u + tb;
+        const uint32_t keys = min_u16x2(upper_halves(x0, x1), 0x06000600u) & 0xFFF8FFF8u;
+        a[i] = dot_u16x2(keys, 0x0010u, tb);
+        a[i + 1] = dot_u16x2(keys, 0x1000u, tb);
     }
     float w[16];
 #pragma unroll
@@ -242,6 +271,91 @@ __device__ __forceinline__ float hp16(const uint32_t *r, uint32_t *pk, float c, 
     return s0 + s1;
 }
 
+// The restart test of a tile: HiF8(T) > lambda  <=>  T >= the midpoint between lambda and the next HiF8 value above it
+// (rounding is monotone, ties go up): 2^-23 | 1.0625 | 2.125 | 3.125 for lambda 0 | 1 | 2 | 3.
+__device__ __forceinline__ float restart_threshold(int lambda)
+{
+    return lambda == 0 ? 1.1920928955078125e-07f : (float)lambda + (lambda == 1 ? 0.0625f : 0.125f);
+}
+// ceil of the row maximum's score; the product was rounded: made sure that no T against it is positive
+__device__ __forceinline__ float int_max(float mx, float c)
+{
+    const float smax = ceilf(mx * c);
+    return fmaf(mx, c, -smax) > 0.f ? smax + 1.f : smax;
+}
+// The thread's n columns of O~, n a multiple of 16, times f.
+__device__ __forceinline__ void rescale_columns(uint32_t o_addr, int n, float f)
+{
+#pragma unroll 1
+    for (int i0 = 0; i0 < n; i0 += 16) {
+        uint32_t o[16];
+        sm100::tmem_ld16(o_addr + i0, o);
+        sm100::tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+        sm100::tmem_st16(o_addr + i0, o);
+    }
+}
+
+// What a thread keeps of its row: m, the running max of Algorithm 1 (integer valued; real valued in the exact and
+// Exp2 modes); m_ref, the max O~ and d are currently expressed against; d, the partial sum of the thread's columns.
+// All rescale factors of Algorithm 1 are exact powers of two, so instead of multiplying O~ by 2^(m_old - m_new)
+// whenever the max moves, a tile's weights are multiplied by 2^e, e = m - m_ref, held as what it adds to the
+// exponents of a packed pair of weights.  O~ is touched only when e has passed 64 and the max moves again.  The
+// threads of a row take identical decisions.
+// The max of a row moves a handful of times over all key tiles, so an 8-bit tile first asks whether it does in any
+// row of the warp, and nothing below is worked out where it does not.
+struct RowState {
+    float m, m_ref, d;
+    uint32_t escale;
+
+    __device__ __forceinline__ void set_scale() { escale = (uint32_t)(int)(m - m_ref) * 0x00800080u; }
+    // A tile in which some row of the warp has a positive T (um: that of the row's maximum mx) or which is restarted.
+    // Moves m to the max that the tile's T are taken against and returns the max after the tile.
+    template <class Rebase>
+    __device__ __forceinline__ float decide(float mx, float c, float um, bool restart_tile, Rebase rebase)
+    {
+        float m_next;
+        if (restart_tile) {
+            m_next = m = fmaxf(m, int_max(mx, c));
+        } else {
+            // delta = max(0, ceil(rowmax T8)); weights 2^T8 * 2^-delta = 2^T8 against the old max.
+            // The tile passed the restart test, so T < 3.125, and ceil(HiF8(T)) only depends on which
+            // rounding midpoints T has reached: 0 below 2^-23 (rounds to 0), else 1 below 1.0625,
+            // else 2 below 2.125, else 3.
+            m_next = m + ((um >= 1.1920928955078125e-07f ? 1.f : 0.f) + (um >= 1.0625f ? 1.f : 0.f) +
+                          (um >= 2.125f ? 1.f : 0.f));
+        }
+        const float kk = m - m_ref;
+        const bool need = kk > 64.f;
+        if (__any_sync(0xffffffffu, need)) {
+            const float f = need ? pow2_int(-kk) : 1.f;
+            rebase(f);
+            d *= f;
+            if (need) m_ref = m;
+        }
+        set_scale();
+        return m_next;
+    }
+    __device__ __forceinline__ void move(float m_next) { m = m_next; set_scale(); }
+    __device__ __forceinline__ void add(float sum) { d += sum * __uint_as_float(0x3F800000u + (escale & 0x7F800000u)); }
+};
+
+// Tables of the softmax warps: the 32-way replicated fast-path table (one global load per entry, copies written with
+// 16-byte stores) and the plain full table.
+__device__ __forceinline__ void fill_attention_tables(uint8_t *rep_table, uint8_t *full_table, int t, int nthreads)
+{
+    float4 *rep = reinterpret_cast<float4 *>(rep_table);
+    for (int e = t; e < kLutRepEntries; e += nthreads) {
+        const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
+        const float4 w4 = make_float4(w, w, w, w);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) rep[e * 8 + i] = w4;
+    }
+    float *full = reinterpret_cast<float *>(full_table);
+    for (int i = t; i < kLutN; i += nthreads) full[i] = g_w0.v[i];
+}
+
 __device__ __forceinline__ float max8(const uint32_t *x)
 {
     return max3(max3(__uint_as_float(x[0]), __uint_as_float(x[1]), __uint_as_float(x[2])),
@@ -297,18 +411,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     const int q_row0 = (b * p.H + h) * p.S + qbase * 128;           // row in the [B*H*S, D] view
     const int kv_row0 = (b * p.Hkv + hk) * p.S;
 
-    // Tables of the softmax warps, built while the first Q / K tiles are on their way: the 32-way replicated
-    // fast-path table (one global load per entry, copies written with 16-byte stores) and the plain full table.
+    // built while the first Q / K tiles are on their way
     auto fill_tables = [&] {
-        float4 *rep = reinterpret_cast<float4 *>(smem + L::kLutRepOff);
-        for (int e = tid; e < kLutRepEntries; e += kTcSoftmaxWarps * 32) {
-            const float w = (e < 16) ? 1.f : g_w0.v[e - 16];
-            const float4 w4 = make_float4(w, w, w, w);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) rep[e * 8 + i] = w4;
-        }
-        float *full = reinterpret_cast<float *>(smem + L::kLutFullOff);
-        for (int i = tid; i < kLutN; i += kTcSoftmaxWarps * 32) full[i] = g_w0.v[i];
+        fill_attention_tables(smem + L::kLutRepOff, smem + L::kLutFullOff, tid, kTcSoftmaxWarps * 32);
     };
 
     // ---- setup --------------------------------------------------------------------------------
@@ -552,18 +657,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
         constexpr bool exact = kMode == BAPS_MODE_EXACT;
         constexpr bool e2e = kMode == BAPS_MODE_E2E_HIF8;
         const bool count_restarts = p.restarts != nullptr && warp == 0;
-        // HiF8(T) > lambda  <=>  T >= the midpoint between lambda and the next HiF8 value above it
-        // (rounding is monotone, ties go up): 2^-23 | 1.0625 | 2.125 | 3.125 for lambda 0 | 1 | 2 | 3.
-        const float over_thr = p.lambda == 0 ? 1.1920928955078125e-07f
-                                             : (float)p.lambda + (p.lambda == 1 ? 0.0625f : 0.125f);
-        // Per query tile t: m, the running max of Algorithm 1 (integer valued; real valued in the exact
-        // and Exp2 modes); m_ref, the max O~ and d are currently expressed against.  All rescale
-        // factors of Algorithm 1 are exact powers of two, so instead of multiplying O~ by
-        // 2^(m_old - m_new) whenever the max moves, the tile's weights are multiplied by
-        // 2^(m~ - m_ref); O~ is touched only if that exponent grows past 64 (or past 8 in the exact
-        // mode, whose factors are not exact).  The four threads of a row take identical decisions; each
-        // keeps the partial sum d of its column quarter.
-        float m[2] = {-INFINITY, -INFINITY}, m_ref[2] = {0.f, 0.f}, d[2] = {0.f, 0.f};
+        const float over_thr = restart_threshold(p.lambda);
+        // per query tile t; O~ and d are rebased past an exponent of 8 in the exact mode, whose factors are not exact
+        RowState st[2] = {{-INFINITY, 0.f, 0.f, 0u}, {-INFINITY, 0.f, 0.f, 0u}};
         int n_restart[2] = {0, 0};
         int k = 0;                               // running task index
         uint32_t r[32];                          // scores of the current task (my quarter row)
@@ -595,113 +691,75 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
             }
             const bool hp = !kExp2 && ((j < nb0) || exact);
             const float g[4] = {max8(&r[0]), max8(&r[8]), max8(&r[16]), max8(&r[24])};
-            float mx;
-            bool restart_tile = false;
-            {
-                const float hm = fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3]));
-                sts_f32(x_addr + 4u * (uint32_t)cq, hm);
-                if (e2e && j >= nb0) {
-                    // The restart decision is tile-wide: does any row have HiF8(T of its maximum) >
-                    // lambda?  The test is monotone, so a row passes it iff one of its quarters does:
-                    // one reducing barrier over all softmax threads gives the verdict and also orders
-                    // the exchange of the quarter maxima.
-                    restart_tile = named_bar_or(5, kTcSoftmaxWarps * 32, fmaf(hm, c, -m[T]) >= over_thr);
-                    if (count_restarts && restart_tile) ++n_restart[T];
-                } else {
-                    named_bar_sync(1 + q4, 128);
-                }
+            const float hm = fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3]));
+            sts_f32(x_addr + 4u * (uint32_t)cq, hm);
+            auto row_max = [&] {
                 const float4 pm = lds_f32x4(x_addr);
-                mx = fmaxf(fmaxf(pm.x, pm.y), fmaxf(pm.z, pm.w));
-            }
+                return fmaxf(fmaxf(pm.x, pm.y), fmaxf(pm.z, pm.w));
+            };
+            auto rebase = [&](float f) {
+                mbar_wait(bar(BD + T), (uint32_t)((j - 1) & 1), s_abort, &g_async_status, 0x330 + T);
+                tc_fence_after_sync();
+                rescale_columns(tmem + lane_sel + 256 + T * D + cq * (D / 4), D / 4, f);
+            };
             // ---- decisions (Algorithm 1: B0 branch / restart test / max update) -----------------
-            // T of the row maximum, formed exactly like every element's T (one FMA)
-            const float um = (hp || kExp2) ? -1.f : fmaf(mx, c, -m[T]);
-            const bool posf = um > 0.f;                       // the row has a positive T
-            const bool any_posf = __any_sync(0xffffffffu, posf);
-            float m_new, mref_w;                    // T of this tile is taken against mref_w
-            if constexpr (kExp2) {
-                // Eq. (2): real-valued running max.  The product was rounded: step the max up by one
-                // unit in the last place if the row maximum's T would come out positive, so that every
-                // T of the tile is <= 0.
-                float smax = mx * c;
-                if (fmaf(mx, c, -smax) > 0.f)
-                    smax = __uint_as_float(__float_as_uint(smax) + (smax >= 0.f ? 1u : 0xFFFFFFFFu));
-                m_new = fmaxf(m[T], smax);
-                mref_w = m_new;
-                if (j > 0) {
-                    // rescale factor 2^(m_old - m_new), 8-bit in and out (not a power of two): O~ and d
-                    // are multiplied for real, once P V of this query tile's previous task is complete.
-                    const float alpha = lds_f32(lut_full + 4u * (uint32_t)w0_index(m[T] - m_new));
-                    if (__any_sync(0xffffffffu, alpha != 1.f)) {
-                        mbar_wait(bar(BD + T), (uint32_t)((j - 1) & 1), s_abort, &g_async_status, 0x330 + T);
-                        tc_fence_after_sync();
-                        const uint32_t o_addr = tmem + lane_sel + 256 + T * D + cq * (D / 4);
-#pragma unroll 1
-                        for (int ch = 0; ch < D / 64; ++ch) {
-                            uint32_t o[16];
-                            tmem_ld16(o_addr + ch * 16, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                            tmem_st16(o_addr + ch * 16, o);
-                        }
-                    }
-                    d[T] *= alpha;
+            bool changed = false, restart_tile = false;
+            float m_next, mref_w;                   // T of this tile is taken against mref_w
+            if (e2e && !hp) {
+                // The restart decision is tile-wide: does any row have HiF8(T of its maximum) >
+                // lambda?  The test is monotone, so a row passes it iff one of its quarters does:
+                // one reducing barrier over all softmax threads gives the verdict and also orders
+                // the exchange of the quarter maxima.  T of the row maximum is formed exactly like every element's
+                // T (one FMA).
+                restart_tile = named_bar_or(5, kTcSoftmaxWarps * 32, fmaf(hm, c, -st[T].m) >= over_thr);
+                const float mx = row_max();
+                const float um = fmaf(mx, c, -st[T].m);
+                changed = restart_tile || __any_sync(0xffffffffu, um > 0.f);
+                m_next = st[T].m;
+                if (changed) {
+                    if (count_restarts && restart_tile) ++n_restart[T];
+                    m_next = st[T].decide(mx, c, um, restart_tile, rebase);
                 }
-                m_ref[T] = m_new;
-            } else if (hp || restart_tile) {
-                float smax = mx * c;
-                if (!exact) {
-                    smax = ceilf(smax);
-                    // the product was rounded: make sure no T against the new max is positive
-                    if (fmaf(mx, c, -smax) > 0.f) smax += 1.f;
-                }
-                m_new = fmaxf(m[T], smax);
-                if (j == 0) m_ref[T] = m_new;
-                mref_w = hp ? m_ref[T] : m_new;
+                mref_w = st[T].m;
             } else {
-                // delta = max(0, ceil(rowmax T8)); weights 2^T8 * 2^-delta = 2^T8 against the old max.
-                // The tile passed the restart test, so T < 3.125, and ceil(HiF8(T)) only depends on which
-                // rounding midpoints T has reached: 0 below 2^-23 (rounds to 0), else 1 below 1.0625,
-                // else 2 below 2.125, else 3.
-                const float delta = (um >= 1.1920928955078125e-07f ? 1.f : 0.f) + (um >= 1.0625f ? 1.f : 0.f) +
-                                    (um >= 2.125f ? 1.f : 0.f);
-                m_new = m[T] + delta;
-                mref_w = m[T];
-            }
-            // ---- rebase O~ and d (rare): only when the exponent against m_ref grows too large -------
-            if constexpr (!kExp2) {
-                const float target = hp ? m_new : mref_w;
-                const float kk = target - m_ref[T];
-                const bool need = (j > 0) && (kk > (exact ? 8.f : 64.f));
-                if (__any_sync(0xffffffffu, need)) {
-                    const float f = need ? (exact ? ex2_approx(-kk) : pow2_int(-kk)) : 1.f;
-                    mbar_wait(bar(BD + T), (uint32_t)((j - 1) & 1), s_abort, &g_async_status, 0x330 + T);
-                    tc_fence_after_sync();
-                    const uint32_t o_addr = tmem + lane_sel + 256 + T * D + cq * (D / 4);
-#pragma unroll 1
-                    for (int ch = 0; ch < D / 64; ++ch) {
-                        uint32_t o[16];
-                        tmem_ld16(o_addr + ch * 16, o);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-                        tmem_st16(o_addr + ch * 16, o);
+                named_bar_sync(1 + q4, 128);
+                const float mx = row_max();
+                if constexpr (kExp2) {
+                    // Eq. (2): real-valued running max.  The product was rounded: step the max up by one
+                    // unit in the last place if the row maximum's T would come out positive, so that every
+                    // T of the tile is <= 0.
+                    float smax = mx * c;
+                    if (fmaf(mx, c, -smax) > 0.f)
+                        smax = __uint_as_float(__float_as_uint(smax) + (smax >= 0.f ? 1u : 0xFFFFFFFFu));
+                    m_next = mref_w = fmaxf(st[T].m, smax);
+                    if (j > 0) {
+                        // rescale factor 2^(m_old - m_new), 8-bit in and out (not a power of two): O~ and d
+                        // are multiplied for real, once P V of this query tile's previous task is complete.
+                        const float alpha = lds_f32(lut_full + 4u * (uint32_t)w0_index(st[T].m - m_next));
+                        if (__any_sync(0xffffffffu, alpha != 1.f)) rebase(alpha);
+                        st[T].d *= alpha;
                     }
-                    d[T] *= f;
-                    if (need) {
-                        m_ref[T] = target;
-                        if (hp) mref_w = target;
+                    st[T].m_ref = m_next;
+                } else {
+                    m_next = fmaxf(st[T].m, exact ? mx * c : int_max(mx, c));
+                    if (j == 0) st[T].m_ref = m_next;
+                    const float kk = m_next - st[T].m_ref;
+                    const bool need = (j > 0) && (kk > (exact ? 8.f : 64.f));
+                    if (__any_sync(0xffffffffu, need)) {
+                        const float f = need ? (exact ? ex2_approx(-kk) : pow2_int(-kk)) : 1.f;
+                        rebase(f);
+                        st[T].d *= f;
+                        if (need) st[T].m_ref = m_next;
                     }
+                    mref_w = st[T].m_ref;
                 }
+                st[T].m = m_next;
+                st[T].escale = 0u;                 // these weights are taken against m_ref (Exp2: against m, with e = 0)
             }
-            // weights are expressed against m_ref: factor 2^e, e = mref_w - m_ref in [0, 64]
-            const float e_f = (hp || kExp2) ? 0.f : (mref_w - m_ref[T]);
-            const int e_i = (int)e_f;                 // 0 .. 64 (the rebase above keeps it there)
-            const uint32_t escale = (uint32_t)e_i * 0x00800080u;
+            const uint32_t escale = st[T].escale;
             // some row of this warp has T > 0 in a tile that was not restarted: the 8-column groups
             // holding those few entries are redone with the full table after the fast path
-            const bool pos_tile = e2e && !hp && !restart_tile && any_posf;      // warp-uniform
+            const bool pos_tile = changed && !restart_tile;                    // warp-uniform
             // ---- weights -> bf16 P over score columns already read; row sum ---------------------------
             float sum = 0.f;
             uint32_t pk[16];
@@ -735,8 +793,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
             tmem_wait_st();
             tc_fence_before_sync();
             mbar_arrive(bar(BP + (k & 1)));       // P is in place: the tensor core's burst may go
-            d[T] += sum * __int_as_float((127 + e_i) << 23);
-            m[T] = m_new;
+            st[T].add(sum);
+            if (changed || (kB0Last && hp)) st[T].move(m_next);
             // the next task's scores travel into registers while the loop turns around
             if (has_next) load_scores(k + 1);
             ++k;
@@ -761,7 +819,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
             // total denominator of the row = the four quarter sums
             // the exchange buffer not used by the task before (that one may still be read by a partner)
             const uint32_t x_addr = xrow + (uint32_t)((k + T) & 1) * 2048u;
-            sts_f32(x_addr + 4u * (uint32_t)cq, d[T]);
+            sts_f32(x_addr + 4u * (uint32_t)cq, st[T].d);
             named_bar_sync(1 + q4, 128);
             const float4 pd = lds_f32x4(x_addr);
             const float dtot = (pd.x + pd.y) + (pd.z + pd.w);
@@ -816,9 +874,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
             }
             if (!good) return;
             if (cq == 0) {
-                if (p.row_m) p.row_m[grow] = m[T];
+                if (p.row_m) p.row_m[grow] = st[T].m;
                 // d is held against m_ref; report it against the final max
-                if (p.row_d) p.row_d[grow] = dtot * (exact ? ex2_approx(m_ref[T] - m[T]) : pow2_int(m_ref[T] - m[T]));
+                if (p.row_d) p.row_d[grow] = dtot * (exact ? ex2_approx(st[T].m_ref - st[T].m) : pow2_int(st[T].m_ref - st[T].m));
             }
             if (count_restarts && lane == 0)
                 p.restarts[(size_t)(b * p.H + h) * p.nq + qi] = n_restart[T];
