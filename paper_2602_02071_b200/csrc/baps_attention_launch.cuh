@@ -1,6 +1,7 @@
 // Host side of the bf16 / 8-bit fused attention: tensor maps, choice of kernel, launch.
 #pragma once
 #include "baps_attention_d64.cuh"
+#include "baps_attention_pair.cuh"
 #include "baps_attention_tc.cuh"
 #include "baps_tma_host.cuh"
 
@@ -71,14 +72,14 @@ static inline baps_status attention_tc_launch(const void *q, const void *k, cons
         if (mode == kExact) return launch_attention<attention_tc_kernel<128, kExact, true, false>, TcLayout<128>::kDynBytes>(a);
         return b0l ? launch_attention<attention_tc_kernel<128, kE2E, true, true>, TcLayout<128>::kDynBytes>(a)
                    : one ? launch_attention<attention_tc_kernel<128, kE2E, true, false, true>, TcLayout<128>::kDynBytes>(a)
-                         : launch_attention<attention_tc_kernel<128, kE2E, true, false, false>, TcLayout<128>::kDynBytes>(a);
+                         : launch_attention<paired_attention_tc_kernel<true>, PairLayout::kDynBytes>(a);
     }
     if (D == 128) {
         if (mode == kExp2m) return launch_attention<attention_tc_kernel<128, kExp2m, false, false>, TcLayout<128>::kDynBytes>(a);
         if (mode == kExact) return launch_attention<attention_tc_kernel<128, kExact, false, false>, TcLayout<128>::kDynBytes>(a);
         return b0l ? launch_attention<attention_tc_kernel<128, kE2E, false, true>, TcLayout<128>::kDynBytes>(a)
                    : one ? launch_attention<attention_tc_kernel<128, kE2E, false, false, true>, TcLayout<128>::kDynBytes>(a)
-                         : launch_attention<attention_tc_kernel<128, kE2E, false, false, false>, TcLayout<128>::kDynBytes>(a);
+                         : launch_attention<paired_attention_tc_kernel<false>, PairLayout::kDynBytes>(a);
     }
     if (mode == kExp2m) return launch_attention<attention_tc_kernel<64, kExp2m, false, false>, TcLayout<64>::kDynBytes>(a);
     if (mode == kExact) return launch_attention<attention_tc_kernel<64, kExact, false, false>, TcLayout<64>::kDynBytes>(a);
