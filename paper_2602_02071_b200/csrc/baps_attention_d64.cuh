@@ -246,6 +246,8 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
             uint64_t s01 = 0ull, s23 = 0ull;
             const float mnv = st.m * 7.52316384526264e-37f, cnv = -c * 7.52316384526264e-37f;     // 2^-120
             const uint64_t cn2 = pack2(cnv, cnv), mn2 = pack2(mnv, mnv);
+            // the 8-column groups that hold a positive T are redone after the fast path
+            const uint32_t pos = changed && !restart_tile ? positive_groups(g, c, st.m) : 0u;
             auto weights = [&](int cc) {
                 uint32_t pk[16];
                 if constexpr (hp) {
@@ -253,14 +255,10 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
                 } else {
                     fast16<false>(&r[0], &pk[0], cn2, mn2, st.escale, tb, s01, s23);
                     fast16<false>(&r[16], &pk[8], cn2, mn2, st.escale, tb, s01, s23);
-                    if (changed && !restart_tile) {
+                    if (pos) {
 #pragma unroll
-                        for (int gg = 0; gg < 4; ++gg) {
-                            const bool gpos = fmaf(cc ? g[4 + gg] : g[gg], c, -st.m) > 0.f;
-                            if (__any_sync(0xffffffffu, gpos))
-                                sum += fix8(&r[gg * 8], &pk[gg * 4], c, st.m, st.escale, lut_full);
-                            __syncwarp();
-                        }
+                        for (int gg = 0; gg < 4; ++gg)
+                            if (pos >> (4 * cc + gg) & 1u) sum += fix8(&r[gg * 8], &pk[gg * 4], c, st.m, lut_full);
                     }
                 }
                 tmem_st16(p_addr + cc * 16, pk);

@@ -265,6 +265,8 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
             const float mnv = kQK8 ? -st.m : st.m * 7.52316384526264e-37f;        // 2^-120
             const float cnv = kQK8 ? c : -c * 7.52316384526264e-37f;
             const uint64_t cn2 = pack2(cnv, cnv), mn2 = pack2(mnv, mnv);
+            // the 8-column groups that hold a positive T are redone after the fast path
+            const uint32_t pos = changed && !restart_tile ? positive_groups(g, c, st.m) : 0u;
             auto weights = [&](int cc) {
                 uint32_t pk[16];
                 if constexpr (hp) {
@@ -272,14 +274,10 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
                 } else {
                     fast16<kQK8>(&r[0], &pk[0], cn2, mn2, st.escale, tb, s01, s23);
                     fast16<kQK8>(&r[16], &pk[8], cn2, mn2, st.escale, tb, s01, s23);
-                    if (changed && !restart_tile) {
+                    if (pos) {
 #pragma unroll
-                        for (int gg = 0; gg < 4; ++gg) {
-                            const bool gpos = fmaf(cc ? g[4 + gg] : g[gg], c, -st.m) > 0.f;
-                            if (__any_sync(0xffffffffu, gpos))
-                                sum += fix8(&r[gg * 8], &pk[gg * 4], c, st.m, st.escale, lut_full);
-                            __syncwarp();
-                        }
+                        for (int gg = 0; gg < 4; ++gg)
+                            if (pos >> (4 * cc + gg) & 1u) sum += fix8(&r[gg * 8], &pk[gg * 4], c, st.m, lut_full);
                     }
                 }
                 tmem_st16(s_addr + cc * 32, pk);

@@ -227,30 +227,46 @@ __device__ __forceinline__ void fast16(const uint32_t *r, uint32_t *pk, uint64_t
     }
 }
 
-// Eight columns of a group that holds a positive T (rows whose maximum rose above the running max
-// in a tile that was not restarted have a few of those; the fast path gave them weight 0).  Only
-// the positive entries are touched: each is looked up in the positive window of the full table
-// (0 < T < 4 because the tile passed the restart test), patched into its half of the packed
-// register and returned as the amount to add to the row sum.  Lanes without a positive entry skip the
-// patch (a plain divergent branch: a warp-wide vote per entry cost more than it saved); the caller
-// reconverges the warp afterwards.
-__device__ __forceinline__ float fix8(const uint32_t *x, uint32_t *pk4, float c, float mref, uint32_t escale,
-                                      uint32_t lut_full)
+// Weight of a positive T (0 < T < 4 because the tile passed the restart test), from the positive window of the full
+// table; 0 for any other T.
+__device__ __forceinline__ float positive_weight(float u, uint32_t lut_pos)
+{
+    const uint32_t key = min(max(__float_as_uint(u) >> 19, (uint32_t)kLutPosLo), (uint32_t)kLutPosHi);
+    float w;
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.gt.f32 p, %1, 0f00000000;\n\t"
+        "mov.f32 %0, 0f00000000;\n\t"
+        "@p ld.shared.f32 %0, [%2];\n\t}"
+        : "=f"(w)
+        : "f"(u), "r"(lut_pos + 4u * key));
+    return w;
+}
+// Eight columns of a group that holds a positive T (rows whose maximum rose above the running max in a tile that was
+// not restarted have a few of those; the fast path gave them weight 0, so theirs is added).  Returns the amount to
+// add to the row sum.  Free of branches: with a divergent branch per element the eight lookups ran one after the
+// other, and since a tile waits for its slowest warp, that, not the number of instructions, was what positive T
+// cost (8 heads x 16384 tokens: 565 us, 470 with them left at weight 0).
+__device__ __forceinline__ float fix8(const uint32_t *x, uint32_t *pk4, float c, float mref, uint32_t lut_full)
 {
     const uint32_t lut_pos = lut_full + 4u * (uint32_t)(kLutNegN - kLutPosLo);
     float add = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float u = fmaf(__uint_as_float(x[i]), c, -mref);
-        if (u > 0.f) {                         // few lanes, if any: the others skip
-            const uint32_t key = min(max(__float_as_uint(u) >> 19, (uint32_t)kLutPosLo), (uint32_t)kLutPosHi);
-            const float w = lds_f32(lut_pos + 4u * key);
-            add += w;
-            const uint32_t half = (__float_as_uint(w) >> 16) + (escale & 0xFFFFu);   // exact in bf16
-            pk4[i >> 1] = (i & 1) ? __byte_perm(pk4[i >> 1], half, 0x5410) : __byte_perm(pk4[i >> 1], half, 0x3254);
-        }
+    for (int i = 0; i < 8; i += 2) {
+        const float w0 = positive_weight(fmaf(__uint_as_float(x[i]), c, -mref), lut_pos);
+        const float w1 = positive_weight(fmaf(__uint_as_float(x[i + 1]), c, -mref), lut_pos);
+        add += w0 + w1;
+        pk4[i >> 1] += upper_halves(w0, w1);                 // exact in bf16
     }
     return add;
+}
+// Which of a warp's groups of eight columns hold a positive T in some row (bit g), from the groups' maxima.
+template <int N>
+__device__ __forceinline__ uint32_t positive_groups(const float (&g)[N], float c, float mref)
+{
+    uint32_t mask = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) mask |= fmaf(g[i], c, -mref) > 0.f ? 1u << i : 0u;
+    return __reduce_or_sync(0xffffffffu, mask);
 }
 
 // High-precision tile (B0, or every tile in the exact mode): P = 2^(S*c - mref) in fp32, rounded
@@ -776,13 +792,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
                 fast16<kTwo>(&r[0], &pk[0], cn2, mn2, escale, tb, s01, s23);
                 fast16<kTwo>(&r[16], &pk[8], cn2, mn2, escale, tb, s01, s23);
                 if (pos_tile) {
+                    const uint32_t groups = positive_groups(g, c, mref_w);
 #pragma unroll
-                    for (int gg = 0; gg < 4; ++gg) {
-                        const bool gpos = fmaf(g[gg], c, -mref_w) > 0.f;
-                        if (__any_sync(0xffffffffu, gpos))
-                            sum += fix8(&r[gg * 8], &pk[gg * 4], c, mref_w, escale, lut_full);
-                        __syncwarp();
-                    }
+                    for (int gg = 0; gg < 4; ++gg)
+                        if (groups >> gg & 1u) sum += fix8(&r[gg * 8], &pk[gg * 4], c, mref_w, lut_full);
                 }
                 float a0, a1, a2, a3;
                 unpack2(s01, a0, a1); unpack2(s23, a2, a3);
