@@ -48,3 +48,14 @@ def test_no_load_asks_for_data_that_never_changes():
     """ld.global.nc (__ldg) may be served from data read before the kernel ahead wrote it."""
     for name, code in CODE.items():
         assert "__ldg(" not in code and "ld.global.nc" not in code, name
+
+
+def test_the_paired_kernel_keeps_the_rules_too():
+    """paired_attention_tc_kernel: the same calls, and a CTA as large as attention_tc_kernel's, so that nothing that uses
+    tensor memory fits beside it."""
+    body = kernel_body("paired_attention_tc_kernel")
+    assert "await_previous_kernel(" in body and "allow_next_kernel()" in body
+    # every role that touches caller memory, or starts a bounded wait, stands behind the wait for the kernel ahead: the
+    # producer before its first load (ahead of the CTA-wide barrier that all other roles pass), the softmax warps at entry
+    assert body.index("await_previous_kernel()") < body.index("tma_load_2d(sbase + L::kQOff") < body.index("__syncthreads()")
+    assert "__launch_bounds__(kTcThreads, 1)" in CODE["baps_attention_pair.cuh"]

@@ -8,6 +8,7 @@ import torch
 import oracle
 from paper_2602_02071_b200 import binding, workloads
 from parity import EPS_REL, gate_attention
+from tile_order import form
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +64,23 @@ def test_fp8_full_size_sampled_and_close_to_the_bf16_path():
     ref16 = binding.baps_attention_fwd_ex(q.cuda(), k.cuda(), v.cuda(), causal=True, block_q=128, block_k=128)
     diff = (st.out_f32 - ref16.out_f32).abs()
     assert float(diff.mean()) < 6e-2 and float(diff.max()) < 2.5
+
+
+@pytest.mark.parametrize("S,causal,lam", [(640, True, 1), (768, True, 2), (256, False, 0)])
+def test_fp8_two_query_tiles_per_cta_agree_with_one(S, causal, lam):
+    """A few heads (one query tile per CTA) and the same heads repeated until the SMs are full several times over
+    (two, an odd one left over at S = 640), outlier keys (restarts): the same decisions, and the same sums but for
+    their order (2^-17, as for bf16 Q / K)."""
+    n = 160
+    assert form(128, 4, S // 128, causal) == "one tile" and form(128, 4 * n, S // 128, causal) == "two tiles"
+    w = workloads.AttnWorkload("t", 1, 4, 2, S, 128, causal, 128, 128, outlier_frac=0.01, seed=400 + S + lam)
+    few, (q, k, v) = _check(w, lam=lam, what=f"fp8 one tile S={S}")
+    (q8, qs, _), (k8, ks, _) = (workloads.quantize_e4m3_tiles(t) for t in (q, k))
+    many = binding.baps_attention_fwd_fp8(*(t.cuda().repeat(n, *[1] * (t.dim() - 1)) for t in (q8, k8, v, qs, ks)),
+                                          causal=causal, lam=lam)
+    assert torch.equal(few.row_m.expand_as(many.row_m), many.row_m)
+    assert torch.equal(few.restarts.expand_as(many.restarts), many.restarts)
+    assert torch.allclose(few.row_d.expand_as(many.row_d), many.row_d, rtol=2.0 ** -17, atol=0)
+    # (a row's outputs are of the size of its largest, and what is left where they cancel is not)
+    scale = few.out_f32.abs().amax(-1, keepdim=True)
+    assert float(((few.out_f32 - many.out_f32).abs() / scale).max()) <= 2.0 ** -17

@@ -54,3 +54,14 @@ def test_the_built_kernels_have_the_registers(split):
     assert len(used) >= 15
     for name, regs in used:
         assert (split.tc_fits if name == "attention_tc_kernel" else split.d64_fits)(int(regs)), (name, regs)
+
+
+def test_the_paired_kernel_takes_its_shares_from_the_split(split):
+    code = open(os.path.join(build.CSRC, "baps_attention_pair.cuh")).read()
+    assert re.findall(r'setmaxnreg\.\w+\.sync\.aligned\.u32 (\S+);" ::"n"\(kTcSplit\.(few|many)\)', code) == [
+        ("%0", "few"), ("%0", "many")]
+    assert code.count("setmaxnreg.") == 2 and "__launch_bounds__(kTcThreads, 1)" in code
+    build.build()
+    log = open(os.path.join(os.path.dirname(build.LIB), "build.log")).read()
+    used = re.findall(r"Compiling entry function '\w*paired_attention_tc_kernel\w*'.*?Used (\d+) registers", log, re.S)
+    assert len(used) == 2 and all(split.tc_fits(int(r)) for r in used)
