@@ -9,8 +9,9 @@
 //               (w / 4) % 2, in two chunks of 32.  Maxima of both chunks, exchange and vote, then the weights of the
 //               second chunk (still in registers) and of the first (read again)
 //   warp 16     TMA producer: Q tiles, then K_0, V_0, K_1, ... through a ring of four 32 KB stages
-//   warp 17     MMA issuer, per tile and stream one burst: P V of tile j, then Q K^T of tile j + 1 into the same
-//               columns (the tensor core runs them in order)
+//   warp 17     MMA issuer, per tile and stream: P V of tile j for the keys of the second chunks as soon as their weights
+//               are there, then for those of the first, and Q K^T of tile j + 1 into the same columns (the tensor
+//               core runs them in order)
 // (warps 18, 19 idle: they complete the warpgroup whose registers go to the softmax warps.)
 // TMEM (512 columns): S_0 | S_1 | O_0 | O_1, 128 columns each; the bf16 weights of column quarter q overwrite columns
 // [32 q, 32 q + 16) of S_t.
@@ -28,8 +29,8 @@ struct PairLayout {
     static constexpr int kLutRepOff = kKvOff + kStages * kTileBytes;
     static constexpr int kLutFullOff = kLutRepOff + kLutRepBytes;
     static constexpr int kBarOff = (kLutFullOff + kLutN * 4 + 15) & ~15;
-    // barriers: q_full, s_full[2], p_full[2], pv_done[2], kv_full[stages], kv_empty[stages]
-    static constexpr int kXchgOff = (kBarOff + (7 + 2 * kStages) * 8 + 15) & ~15;      // float xchg[2 tiles][2][128][2]
+    // barriers: q_full, s_full[2], p_full[2][2], pv_done[2], kv_full[stages], kv_empty[stages]
+    static constexpr int kXchgOff = (kBarOff + (9 + 2 * kStages) * 8 + 15) & ~15;      // float xchg[2 tiles][2][128][2]
     static constexpr int kMiscOff = kXchgOff + 2 * 2 * 128 * 2 * 4;                    // tmem base, abort
     static constexpr int kDynBytes = kMiscOff + 16 + 1024;                             // slack for 1024-byte alignment
 };
@@ -46,8 +47,8 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t sbase = smem_u32(smem);
     auto bar = [&](int i) { return sbase + L::kBarOff + 8u * (uint32_t)i; };
-    // q_full | s_full[t] | p_full[t] | pv_done[t] | kv_full[stage] | kv_empty[stage]
-    constexpr int BQ = 0, BS = 1, BP = 3, BD = 5, BKF = 7, BKE = 7 + L::kStages;
+    // q_full | s_full[t] | p_full[2 t + half of the weights] | pv_done[t] | kv_full[stage] | kv_empty[stage]
+    constexpr int BQ = 0, BS = 1, BP = 3, BD = 7, BKF = 9, BKE = 9 + L::kStages;
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::kMiscOff);
     volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L::kMiscOff + 4);
 
@@ -83,7 +84,8 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
     if (warp == 16) {
         if (lane == 0) {
             mbar_init(bar(BQ), 1);
-            for (int t = 0; t < 2; ++t) { mbar_init(bar(BS + t), 1); mbar_init(bar(BP + t), 8); mbar_init(bar(BD + t), 1); }
+            for (int t = 0; t < 2; ++t) { mbar_init(bar(BS + t), 1); mbar_init(bar(BD + t), 1); }
+            for (int i = 0; i < 4; ++i) mbar_init(bar(BP + i), 8);
             for (int s = 0; s < L::kStages; ++s) { mbar_init(bar(BKF + s), 1); mbar_init(bar(BKE + s), 1); }
             mbar_fence_init();
             await_previous_kernel();
@@ -150,13 +152,15 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
                 mma_commit(bar(BS + t));
                 if (t == (j < j1 ? 1 : 0)) mma_commit(bar(BKE + stage_of(2 * j)));         // the last that reads K_j
             };
-            auto mma_pv = [&](int t, int j) {
+            // O_t += P V_j over the keys of one half of the weights: 32-column quarters 1 and 3 (first), then 0 and 2
+            auto mma_pv = [&](int t, int j, int half) {
                 const uint32_t vd = sdesc_lo(sbase + L::kKvOff + stage_of(2 * j + 1) * L::kTileBytes, 16384);
                 const uint32_t od = tmem + 256 + t * D, pd = tmem + t * 128;
-                const uint32_t acc0 = j > 0 ? 1u : 0u;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    mma_ts_lo(od, pd + (ks >> 1) * 32 + (ks & 1) * 8, vd + ks * 128, idesc_pv, ks > 0 ? 1u : acc0);
+                for (int i = 0; i < 4; ++i) {
+                    const int quarter = (i >> 1) * 2 + 1 - half, ks = 2 * quarter + (i & 1);
+                    mma_ts_lo(od, pd + quarter * 32 + (i & 1) * 8, vd + ks * 128, idesc_pv, half || i || j > 0 ? 1u : 0u);
+                }
             };
             const bool leader = elect_one();
             bool ok = wait_all(bar(BQ), 0, 0x200) && wait_all(bar(BKF), 0, 0x210);
@@ -175,11 +179,16 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
                 for (int t = 0; ok && t < 2; ++t) {
                     const int jt = t ? j1 : j0;
                     if (j >= jt) continue;
-                    ok = wait_all(bar(BP + t), (uint32_t)(j & 1), 0x230 + t);
+                    ok = wait_all(bar(BP + 2 * t), (uint32_t)(j & 1), 0x230 + t);
+                    if (!ok) break;
+                    tc_fence_after_sync();
+                    if (leader) mma_pv(t, j, 0);
+                    __syncwarp();
+                    ok = wait_all(bar(BP + 2 * t + 1), (uint32_t)(j & 1), 0x232 + t);
                     if (!ok) break;
                     tc_fence_after_sync();
                     if (leader) {
-                        mma_pv(t, j);
+                        mma_pv(t, j, 1);
                         if (j + 1 < jt) mma_qk(t, j + 1);
                         mma_commit(bar(BD + t));
                         if (t == (j < j1 ? 1 : 0)) mma_commit(bar(BKE + stage_of(2 * j + 1)));
@@ -221,20 +230,25 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
             mbar_wait(bar(BS + t), (uint32_t)(j & 1), s_abort, &g_async_status, 0x300 + t);
             tc_fence_after_sync();
             // ---- maxima of my 64 columns, exchange with the partner thread, tile-wide vote ----------------
-            auto load_chunk = [&](int cc) {
-                tmem_ld32(s_addr + cc * 32, r);
-                tmem_wait_ld();
+            auto mask_chunk = [&](uint32_t (&x)[32], int cc) {
                 if (diag) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = (ch * 64 + cc * 32 + i > row) ? 0xFF800000u : r[i];
+                    for (int i = 0; i < 32; ++i) x[i] = (ch * 64 + cc * 32 + i > row) ? 0xFF800000u : x[i];
                 }
             };
-            load_chunk(0);
+            {
+                // (both chunks on their way at once: nothing else is in registers yet)
+                uint32_t x[32];
+                tmem_ld32(s_addr, x);
+                tmem_ld32(s_addr + 32, r);
+                tmem_wait_ld();
+                mask_chunk(x, 0);
+                mask_chunk(r, 1);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) g[i] = max8(&r[8 * i]);
-            load_chunk(1);
+                for (int i = 0; i < 4; ++i) g[i] = max8(&x[8 * i]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) g[4 + i] = max8(&r[8 * i]);
+                for (int i = 0; i < 4; ++i) g[4 + i] = max8(&r[8 * i]);
+            }
             const float hm = max3(max3(g[0], g[1], g[2]), max3(g[3], g[4], g[5]), fmaxf(g[6], g[7]));
             sts_f32(x_addr + 4u * (uint32_t)ch, hm);
             bool restart_tile = false;
@@ -282,13 +296,19 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
                 }
                 tmem_st16(s_addr + cc * 32, pk);
             };
+            auto arrive = [&](int half) {
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(BP + 2 * t + half));
+            };
             weights(1);
-            load_chunk(0);
+            arrive(0);                                    // the tensor core starts on the keys of the second chunks
+            tmem_ld32(s_addr, r);
+            tmem_wait_ld();
+            mask_chunk(r, 0);
             weights(0);
-            tmem_wait_st();
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(BP + t));      // P is in place: the tensor core's burst may go
+            arrive(1);                                    // all of P is in place
             if constexpr (!hp) {
                 float a0, a1, a2, a3;
                 unpack2(s01, a0, a1); unpack2(s23, a2, a3);

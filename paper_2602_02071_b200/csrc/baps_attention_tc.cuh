@@ -599,14 +599,17 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
                 mma_commit(bar(BS + (k & 1)));
             };
             // O_t += P V_j with P in S buffer (k & 1): the weights of keys 16 ks .. 16 ks + 15 sit at
-            // columns 32 (ks / 2) + 8 (ks % 2) of the buffer (issuing lane only)
+            // columns 32 (ks / 2) + 8 (ks % 2) of the buffer (issuing lane only; the keys in the order of
+            // paired_attention_tc_kernel, so that both add up alike)
             auto mma_pv = [&](int t, int j, int k) {
                 const uint32_t vd = sdesc_lo(sbase + L::kKvOff + kv_stage(2 * j + 1) * L::kTileBytes, 16384);
                 const uint32_t od = tmem + 256 + t * D, pd = tmem + (k & 1) * 128;
                 const uint32_t acc0 = j > 0 ? 1u : 0u;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    mma_ts_lo(od, pd + (ks >> 1) * 32 + (ks & 1) * 8, vd + ks * 128, idesc_pv, ks > 0 ? 1u : acc0);
+                for (int i = 0; i < 8; ++i) {
+                    const int ks = (i >> 1 & 1) * 4 + (i < 4 ? 2 : 0) + (i & 1);    // column quarters 1, 3, 0, 2
+                    mma_ts_lo(od, pd + (ks >> 1) * 32 + (ks & 1) * 8, vd + ks * 128, idesc_pv, i > 0 ? 1u : acc0);
+                }
             };
             const bool leader = elect_one();
             if (ok && J > 0) {
