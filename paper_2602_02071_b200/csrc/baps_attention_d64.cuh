@@ -167,8 +167,10 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
                     const uint32_t vd = sdesc_lo(sbase + L::kKvOff + stage_of(2 * j + 1) * L::kTileBytes, 16384);
                     const uint32_t acc0 = j > 0 ? 1u : 0u;
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        mma_ts_lo(tmem + 192, tmem + 128 + ks * 8, vd + ks * 128, idesc_pv, ks > 0 ? 1u : acc0);
+                    for (int i = 0; i < 8; ++i) {
+                        const int ks = (i >> 1 & 1) * 4 + (i < 4 ? 2 : 0) + (i & 1);      // as in attention_tc_kernel
+                        mma_ts_lo(tmem + 192, tmem + 128 + ks * 8, vd + ks * 128, idesc_pv, i > 0 ? 1u : acc0);
+                    }
                     mma_commit(bar(BD));
                     mma_commit(bar(BKE + stage_of(2 * j + 1)));
                 }
