@@ -205,20 +205,25 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
             mbar_wait(bar(BS), (uint32_t)(j & 1), s_abort, &g_async_status, 0x300);
             tc_fence_after_sync();
             // ---- maxima of my 64 columns, exchange with the partner thread, tile-wide vote ----------------
-            auto load_chunk = [&](int cc) {
-                tmem_ld32(s_addr + cc * 32, r);
-                tmem_wait_ld();
+            auto mask_chunk = [&](uint32_t (&x)[32], int cc) {
                 if (diag) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = (ch * 64 + cc * 32 + i > row) ? 0xFF800000u : r[i];
+                    for (int i = 0; i < 32; ++i) x[i] = (ch * 64 + cc * 32 + i > row) ? 0xFF800000u : x[i];
                 }
             };
-            load_chunk(0);
+            {
+                // (both chunks on their way at once: nothing else is in registers yet)
+                uint32_t x[32];
+                tmem_ld32(s_addr, x);
+                tmem_ld32(s_addr + 32, r);
+                tmem_wait_ld();
+                mask_chunk(x, 0);
+                mask_chunk(r, 1);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) g[i] = max8(&r[8 * i]);
-            load_chunk(1);
+                for (int i = 0; i < 4; ++i) g[i] = max8(&x[8 * i]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) g[4 + i] = max8(&r[8 * i]);
+                for (int i = 0; i < 4; ++i) g[4 + i] = max8(&r[8 * i]);
+            }
             const float hm = max3(max3(g[0], g[1], g[2]), max3(g[3], g[4], g[5]), fmaxf(g[6], g[7]));
             sts_f32(x_addr + 4u * (uint32_t)ch, hm);
             bool restart_tile = false;
@@ -271,7 +276,9 @@ attention_d64_kernel(const __grid_constant__ CUtensorMap mq, const __grid_consta
                 tc_fence_after_sync();
             }
             weights(1);
-            load_chunk(0);
+            tmem_ld32(s_addr, r);
+            tmem_wait_ld();
+            mask_chunk(r, 0);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(BF));          // the scores have been read for the last time
