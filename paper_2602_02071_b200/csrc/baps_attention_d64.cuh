@@ -19,6 +19,9 @@
 // Measured against that kernel with two query tiles per CTA (heads x tokens): 512 x 1024 bidirectional 351 -> 330 us,
 // 64 x 8192 causal 1233 -> 1101, 24 x 2048 causal 46.2 -> 42.8 on unit-Gaussian inputs; with a per-token key bias
 // (more restarts and positive T) 512 x 1024 342 -> 313.  Small grids keep that kernel (two_ctas_per_sm).
+// Since then: keys two at a time and decisions only where a max moves (RowState) 64 x 8192 1115 -> 1046 us, 512 x 1024 348
+// -> 335; positive T without branches 1045 -> 1001, 335 -> 318; both chunks requested at once 1010 -> 1001, 321 -> 317.  P V in
+// two halves, as in paired_attention_tc_kernel, is slower here (1030, 326): Q K^T of the next tile does not wait for it.
 #pragma once
 #include "baps_attention_tc.cuh"
 

@@ -17,6 +17,14 @@
 // [32 q, 32 q + 16) of S_t.
 // The arithmetic, the bounded waits and the way every role ends after an expired wait are those of
 // attention_tc_kernel; only the row sum is added up in another order (two partial sums per row, not four).
+//
+// What bounds it: the chain of a stream, not a pipe.  A stream takes 3900 cycles per tile (two tiles per SM in that
+// time; the tensor core needs 1024 for one): from its scores to its weights 2500, with two warps per scheduler and
+// stream that do not cover the latency of the lookups, then P V and Q K^T.  Measured against sixteen warps on one tile
+// after the other (attention_tc_kernel with two query tiles; causal, heads x tokens): 8 / 2 x 16384 614 -> 539 us,
+// 64 / 16 x 8192 1250 -> 1092, 64 / 16 x 2048 116 -> 111; bidirectional 128 / 32 x 2048 354 -> 317.  Of that, at the first
+// of these, P V in two halves 559 -> 540, both chunks requested at once 559 -> 538, the two together 539.  The lookups
+// of 32 columns have to be in flight together: sixteen at a time in a rolled loop took 609 to 641.
 #pragma once
 #include "baps_attention_tc.cuh"
 
