@@ -1,5 +1,7 @@
 // Fused BAPS attention forward on the 5th-generation tensor cores (tcgen05, sm_100a).
 //
+// (Algorithm 1 with two query tiles per CTA is paired_attention_tc_kernel's; this kernel serves small grids, B0 = {first,
+// last} and the exact and Exp2 modes, and holds what all of them share.)
 // One CTA owns two consecutive 128-row query tiles (t = 0, 1; small grids: one, see one_tile_per_cta) of one
 // (batch, head) and walks the key tiles j in increasing order (Algorithm 1: tile 0 is the high-precision set B0, all later
 // tiles are 8-bit tiles).  The unit of work is a task (t, j): S = Q_t K_j^T, softmax bookkeeping
