@@ -42,18 +42,18 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # kernel, and the fraction of cycles its tensor pipe was active (a clock-independent counter).
 # None where no capture of that workload exists.
 NCU_CAPTURES = {
-    # profiles/attention_tc_kernel_c5_long_context_dram.txt: one launch of the full workload
-    # (404.1 MB read + 239.3 MB written, 44.0 % of cycles)
-    "c5_long_context": {"traffic": 643.4e6, "tensor_pipe_active_pct": 44.0},
-    # profiles/attention_tc_kernel_c2_llm_prefill_mha.txt: 145.2 MB read + 14.3 MB written
-    "c2_llm_prefill_mha": {"traffic": 159.6e6, "tensor_pipe_active_pct": 37.6},
+    # profiles/paired_attention_tc_kernel_c5_long_context_dram.txt: one launch of the full workload
+    # (405.4 MB read + 235.5 MB written, 52.7 % of cycles)
+    "c5_long_context": {"traffic": 640.9e6, "tensor_pipe_active_pct": 52.7},
+    # profiles/paired_attention_tc_kernel_c2_llm_prefill_mha.txt: 143.3 MB read + 13.7 MB written
+    "c2_llm_prefill_mha": {"traffic": 157.0e6, "tensor_pipe_active_pct": 43.3},
 }
 
 # Thread instructions per score element of the fused kernels, from smsp__inst_executed.sum of the committed
-# captures (profiles/attention_tc_kernel_long_causal_s16384.txt: 12.18; configuration 2 with its outlier keys 12.41;
-# profiles/attention_d64_kernel_vit_b8_s1024.txt: 12.04), and the issue peak of the part: 148 SMs x 4 schedulers x
+# captures (profiles/paired_attention_tc_kernel_long_causal_s16384.txt: 9.24; configuration 2 with its outlier keys
+# 9.64; profiles/attention_d64_kernel_vit_b8_s1024.txt: 11.13), and the issue peak of the part: 148 SMs x 4 schedulers x
 # 32 lanes per clock.
-INSTR_PER_SCORE = {128: 12.2, 64: 12.0}
+INSTR_PER_SCORE = {128: 9.2, 64: 11.1}
 ISSUE_LANES_PER_CLOCK = 148 * 4 * 32
 
 
@@ -590,7 +590,7 @@ def main():
         "tensor_pipe_active_pct_ncu": cap.get("tensor_pipe_active_pct"),
         "traffic": cap.get("traffic"),
         "algorithmic_bytes": float(2 * (2 * w.B * w.H + 2 * w.B * w.Hkv) * w.S * w.D),
-        "kernel": "attention_d64_kernel" if w.D == 64 else "attention_tc_kernel<128, Algorithm 1>", "best_ms": float(np.min(times)),
+        "kernel": "attention_d64_kernel" if w.D == 64 else "paired_attention_tc_kernel<false>", "best_ms": float(np.min(times)),
         "median_ms": float(np.median(times)),
         "ms_x_sm_mhz": kernel_ms * clocks["sm_mhz"] if clocks["sm_mhz"] else None,
         "issue_roofline": issue_roofline(w, kernel_ms, clocks["sm_mhz"]),
