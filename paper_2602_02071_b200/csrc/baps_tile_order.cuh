@@ -9,17 +9,19 @@
 
 namespace baps {
 
-// One query tile per CTA or two?  Two share the K / V stream and the set-up of the CTA, and a task (one score
-// tile, 1.35 us) waits less on the one before it; one halves the chain of tasks that the longest CTA walks
-// through, which is what a grid that does not fill the SMs several times over takes.  Estimate of both in units
-// of a two-tile task, SMs filled longest CTA first: the longest CTA or the average load of an SM, whichever is
-// larger (all CTAs of a bidirectional problem are equally long: whole waves).  Besides its tasks a CTA costs
-// kFixedTwo / kFixedOne (set-up, first scores, epilogues).  Measured, two tiles -> one (D = 128, causal, heads x
-// tokens): 4 x 512 15.8 -> 11.4 us, 8 x 4096 90.8 -> 58.1, 32 x 1024 28.8 -> 23.7, 1 x 16384 326 -> 215; and
-// where two stay: 16 x 4096 90.6 -> 111, 32 x 2048 53.7 -> 67, 4 x 32768 1190 -> 1501.
+// One query tile per CTA or two?  Two share the K / V stream and the set-up of the CTA, and one of them works while the
+// other waits (a task, one score tile, takes 1.08 us of a CTA with two against 1.7 of a CTA with one); one halves the
+// chain of tasks that the longest CTA walks through, which is what a grid that does not fill the SMs several times over
+// takes.  Estimate of both in units of a two-tile task, SMs filled longest CTA first: the longest CTA or the average load of
+// an SM, whichever is larger (all CTAs of a bidirectional problem are equally long: whole waves).  Besides its tasks a
+// CTA costs kFixedTwo / kFixedOne (set-up, first scores, epilogues).  The constants are the middle of those that choose the
+// faster form at all of 52 sizes from 4 x 512 to 4 x 32768 (heads x tokens, D = 128).  Measured, one tile / two tiles,
+// causal: 16 x 512 10.0 / 13.8 us, 32 x 1024 22.6 / 24.7, 16 x 2048 33.6 / 43.3, 8 x 4096 57.0 / 79.1, 1 x 16384 219 / 274; and where
+// two are taken: 64 x 512 17.5 / 15.4, 24 x 2048 51.8 / 44.0, 12 x 4096 89.8 / 78.4, 8 x 8192 206 / 145, 2 x 32768 788 / 523;
+// bidirectional 16 x 512 10.8 / 14.8, 8 x 2048 31.3 / 42.4, and 24 x 2048 90.3 / 83.9, 12 x 4096 169 / 154.
 inline bool one_tile_per_cta(long long heads, int nq, bool causal, int num_sms)
 {
-    constexpr double kFixedTwo = 4.5, kFixedOne = 3.5, kTaskOne = 1.25;
+    constexpr double kFixedTwo = 4.5, kFixedOne = 4.0, kTaskOne = 1.35;
     const long long ctas2 = heads * ((nq + 1) / 2), ctas1 = heads * nq;
     const double longest1 = kTaskOne * nq + kFixedOne, longest2 = (causal || nq == 1 ? 2 * nq - 1 : 2 * nq) + kFixedTwo;
     double t1, t2;
