@@ -1,0 +1,62 @@
+"""GPU parity of the fused attention where its number formats end: a max that rounds to zero from below, in every form of
+the kernel."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2602_02071_b200 import binding
+from tile_order import form
+
+pytestmark = pytest.mark.gpu
+
+# D, copies of two heads, the form of the kernel that this grid takes
+FORMS = [(128, 1, "one tile"), (128, 80, "two tiles"), (64, 1, "one tile"), (64, 160, "two CTAs per SM")]
+
+
+def _score_keys(scores, D):
+    """Keys [2, S, D] whose base-2 score against every query with a 1 in column 0 is scores[key]."""
+    k = torch.zeros(2, scores.numel(), D)
+    k[..., 0] = scores * math.sqrt(D) / 1.4426950408889634
+    return k.bfloat16()
+
+
+def _run(q, k, v, n, want_form, causal, lam=1):
+    """Two heads [2, S, D] repeated n times; the copies give the same bits.  -> statistics of one copy"""
+    H, S, D = q.shape
+    assert form(D, H * n, S // 128, causal) == want_form
+    st = binding.baps_attention_fwd_ex(*(t[None].cuda().repeat(n, 1, 1, 1) for t in (q, k, v)), causal=causal,
+                                       block_q=128, block_k=128, lam=lam)
+    binding.poll_async_error()
+    for t in (st.out, st.out_f32, st.row_m, st.row_d, st.restarts):
+        assert torch.equal(t.nan_to_num(9e9), t[:1].nan_to_num(9e9).expand_as(t))
+    return [t[0].float().cpu() for t in (st.out, st.out_f32, st.row_m, st.row_d, st.restarts)]
+
+
+def _oracle(q, k, v, causal, lam=1):
+    r = oracle.attention(*(t[None].float().numpy() for t in (q, k, v)), causal=causal, block_q=128, block_k=128, lam=lam)
+    return r, tuple(x.reshape(q.shape[:2] + x.shape[2:]) for x in (r.out, r.row_m, r.row_d))
+
+
+@pytest.mark.parametrize("first", [[-0.5], [-5.5, -0.5]])
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("D,n,want_form", FORMS)
+def test_a_max_that_rounds_up_to_zero(D, n, want_form, causal, first):
+    """The largest score so far lies in (-1, 0), in the first tile or after a restart, so that the max is zero; the scores
+    of all later keys are zero exactly (padding): T = 0, weight 1."""
+    S = 640
+    g = torch.Generator().manual_seed(D)
+    q = torch.randn(2, S, D, generator=g).bfloat16()
+    q[..., 0] = 1.0
+    scores = torch.zeros(S)
+    scores[:128 * len(first)] = torch.tensor(first).repeat_interleave(128)
+    k = _score_keys(scores, D)
+    v = (torch.randn(2, S, D, generator=g) + (torch.arange(S) // 128)[:, None]).bfloat16()
+    out, out_f32, row_m, row_d, restarts = _run(q, k, v, n, want_form, causal)
+    ref, (want, want_m, want_d) = _oracle(q, k, v, causal)
+    assert np.array_equal(row_m.numpy(), want_m) and np.array_equal(restarts.numpy().ravel(), ref.restarts)
+    # all scores but the first tile's sit on table entries; those of the first tile have bf16 weights
+    assert np.allclose(row_d.numpy(), want_d, rtol=2.0 ** -8, atol=0)
+    assert np.abs(out_f32.numpy() - want).max() <= 1e-2
