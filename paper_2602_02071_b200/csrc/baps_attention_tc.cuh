@@ -295,12 +295,12 @@ __device__ __forceinline__ float restart_threshold(int lambda)
 {
     return lambda == 0 ? 1.1920928955078125e-07f : (float)lambda + (lambda == 1 ? 0.0625f : 0.125f);
 }
-// ceil of the row maximum's score; the product was rounded: made sure that no T against it is positive.  (+ 0: ceilf gives
-// -0 for scores in (-1, 0), and against that the key of a score of exactly 0 would be that of -0, a positive T's.)
+// ceil of the row maximum's score; the product was rounded: made sure that no T against it is positive.  Never -0, which
+// ceilf gives for scores in (-1, 0): against that the key of a score of exactly 0 would be that of -0, a positive T's.
 __device__ __forceinline__ float int_max(float mx, float c)
 {
-    const float smax = ceilf(mx * c) + 0.f;
-    return fmaf(mx, c, -smax) > 0.f ? smax + 1.f : smax;
+    const float smax = ceilf(mx * c);
+    return smax + (fmaf(mx, c, -smax) > 0.f ? 1.f : 0.f);
 }
 // The thread's n columns of O~, n a multiple of 16, times f.
 __device__ __forceinline__ void rescale_columns(uint32_t o_addr, int n, float f)
