@@ -32,15 +32,17 @@ namespace baps {
 // (integer valued, or -inf before block 0) and the block's largest logit xmax (base-2 score
 // xmax * log2(e)), return the new max.  *restart is set when the restart branch was taken.
 // T of the maximum is formed exactly as for every other element (one fused multiply-add).
+// (ceilf + 0: never -0, which ceilf gives for scores in (-1, 0); against that the table key of a logit of exactly 0 would
+// be that of -0, a positive T's.)
 __device__ __forceinline__ float row_block_update(float m, float xmax, bool first, int lambda,
                                                   bool *restart, float *delta)
 {
     *restart = false; *delta = 0.f;
-    if (first) return fmaxf(m, ceilf(xmax * kLog2e));
+    if (first) return fmaxf(m, ceilf(xmax * kLog2e) + 0.f);
     const float u = fmaf(xmax, kLog2e, -m);
     if (u <= 0.f) return m;                     // T8 <= 0: no restart, delta = 0 (the common case)
     const float t8 = hif8_round(u);
-    if (t8 > (float)lambda) { *restart = true; return fmaxf(m, ceilf(xmax * kLog2e)); }
+    if (t8 > (float)lambda) { *restart = true; return fmaxf(m, ceilf(xmax * kLog2e) + 0.f); }
     const float d = fmaxf(0.f, ceilf(t8));
     *delta = d;
     return m + d;
