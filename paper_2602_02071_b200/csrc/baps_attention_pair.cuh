@@ -268,7 +268,7 @@ paired_attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
             bool changed = false;                 // the max moves in some row of the warp (with or without a restart)
             float m_next = st.m;
             if constexpr (hp) {
-                st.m = st.m_ref = m_next = int_max(mx, c);
+                st.m = st.m_ref = m_next = fmaxf(st.m, int_max(mx, c));      // -inf for a row of NaN
             } else {
                 const float um = fmaf(mx, c, -st.m);
                 changed = restart_tile || __any_sync(0xffffffffu, um > 0.f);

@@ -60,3 +60,25 @@ def test_a_max_that_rounds_up_to_zero(D, n, want_form, causal, first):
     # all scores but the first tile's sit on table entries; those of the first tile have bf16 weights
     assert np.allclose(row_d.numpy(), want_d, rtol=2.0 ** -8, atol=0)
     assert np.abs(out_f32.numpy() - want).max() <= 1e-2
+
+
+@pytest.mark.parametrize("D,n,want_form", FORMS)
+def test_rows_without_a_score_keep_the_max_of_no_key(D, n, want_form):
+    """A query row that holds a NaN has no scores: its output is NaN, its max that of no key (-inf), and no other row, max
+    or restart count notices (the row is compared with one of zeros, which never votes for a restart either)."""
+    S = 512
+    g = torch.Generator().manual_seed(D + 1)
+    q, k, v = (torch.randn(2, S, D, generator=g).bfloat16() for _ in range(3))
+    k[:, 7::100] *= 8                                                   # restarts
+    rows = [5, 200, S - 1]
+    q[:, rows] = 0.0
+    plain = _run(q, k, v, n, want_form, False)
+    q[:, rows, 3] = float("nan")
+    got = _run(q, k, v, n, want_form, False)
+    others = [r for r in range(S) if r not in rows]
+    for a, b in zip(plain[:4], got[:4]):
+        assert torch.equal(a[:, others], b[:, others])
+    assert torch.equal(plain[4], got[4]) and int(got[4].sum()) > 0
+    for t in (got[0], got[1], got[3]):
+        assert torch.isnan(t[:, rows]).all()
+    assert (got[2][:, rows] == -float("inf")).all()
