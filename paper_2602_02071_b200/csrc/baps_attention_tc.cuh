@@ -320,8 +320,8 @@ __device__ __forceinline__ void rescale_columns(uint32_t o_addr, int n, float f)
 // Exp2 modes); m_ref, the max O~ and d are currently expressed against; d, the partial sum of the thread's columns.
 // All rescale factors of Algorithm 1 are exact powers of two, so instead of multiplying O~ by 2^(m_old - m_new)
 // whenever the max moves, a tile's weights are multiplied by 2^e, e = m - m_ref, held as what it adds to the
-// exponents of a packed pair of weights.  O~ is touched only when e has passed 64 and the max moves again.  The
-// threads of a row take identical decisions.
+// exponents of a packed pair of weights.  O~ is touched only when the max moves and e has passed 61: a move without a
+// restart adds 3 at most, so no weight is multiplied by more than 2^64.  The threads of a row take identical decisions.
 // The max of a row moves a handful of times over all key tiles, so an 8-bit tile first asks whether it does in any
 // row of the warp, and nothing below is worked out where it does not.
 struct RowState {
@@ -346,7 +346,7 @@ struct RowState {
                           (um >= 2.125f ? 1.f : 0.f));
         }
         const float kk = m - m_ref;
-        const bool need = kk > 64.f;
+        const bool need = kk > 61.f;
         if (__any_sync(0xffffffffu, need)) {
             const float f = need ? pow2_int(-kk) : 1.f;
             rebase(f);

@@ -82,3 +82,23 @@ def test_rows_without_a_score_keep_the_max_of_no_key(D, n, want_form):
     for t in (got[0], got[1], got[3]):
         assert torch.isnan(t[:, rows]).all()
     assert (got[2][:, rows] == -float("inf")).all()
+
+
+@pytest.mark.parametrize("D,n,want_form", FORMS)
+def test_weights_stay_in_range_until_the_output_is_rebased(D, n, want_form):
+    """The row maximum rises by three per tile up to 66, then stays: O~ and d are rebased before weights of 2^66 meet
+    them.  V of 2^54 does not overflow (the sum over the keys of a tile adds 7 to the exponent, 2^64 times that is
+    2^125), with 2^66 it would."""
+    tiles = 30
+    S = 128 * tiles
+    g = torch.Generator().manual_seed(D + 2)
+    q = torch.zeros(2, S, D).bfloat16()
+    q[..., 0] = 1.0
+    level = torch.tensor([0.0] + [3.0 * min(t, 22) - (0.3 if t <= 22 else 0.5) for t in range(1, tiles)])
+    k = _score_keys(level.repeat_interleave(128), D)
+    v = (torch.rand(2, S, D, generator=g) * 0.5 + 0.5).bfloat16()
+    out, out_f32, row_m, row_d, restarts = _run(q, k, v * 2.0 ** 54, n, want_form, False, lam=3)
+    ref, (want, want_m, want_d) = _oracle(q, k, v, False, lam=3)
+    assert np.array_equal(row_m.numpy(), want_m) and (want_m == 66).all() and not restarts.any()
+    assert np.allclose(row_d.numpy(), want_d, rtol=2.0 ** -8, atol=0)
+    assert np.abs(out_f32.numpy() * 2.0 ** -54 - want).max() <= 1e-2

@@ -329,7 +329,7 @@ def test_two_query_tiles_per_cta_against_the_oracle(S, causal, lam):
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("D,want_form", [(128, "two tiles"), (64, "two CTAs per SM")])
 def test_rising_max_rebases_the_output(D, want_form, causal):
-    """The row maximum rises by more than five with every key tile, past the exponent of 64 at which O~ and d are
+    """The row maximum rises by more than five with every key tile, past the exponent at which O~ and d are
     rebased (its last value against its first is asserted), on grids that take the forms of the long prefills."""
     S, H = 2048, 2
     w = workloads.AttnWorkload("rising", 1, H, H, S, D, causal, 128, 128)
