@@ -1,5 +1,5 @@
-"""GPU parity of the fused attention where its number formats end: a max that rounds to zero from below, in every form of
-the kernel."""
+"""GPU parity of the fused attention where its number formats end, in every form of the kernel: a max that rounds to zero
+from below, rows of NaN, weights near the largest factor, scores of -inf and +inf."""
 import math
 
 import numpy as np
@@ -7,7 +7,8 @@ import pytest
 import torch
 
 import oracle
-from paper_2602_02071_b200 import binding
+from paper_2602_02071_b200 import binding, workloads
+from parity import EPS_REL, gate_attention
 from tile_order import form
 
 pytestmark = pytest.mark.gpu
@@ -102,3 +103,68 @@ def test_weights_stay_in_range_until_the_output_is_rebased(D, n, want_form):
     assert np.array_equal(row_m.numpy(), want_m) and (want_m == 66).all() and not restarts.any()
     assert np.allclose(row_d.numpy(), want_d, rtol=2.0 ** -8, atol=0)
     assert np.abs(out_f32.numpy() * 2.0 ** -54 - want).max() <= 1e-2
+
+
+@pytest.mark.parametrize("D,n,want_form", FORMS)
+def test_scores_of_minus_infinity_have_no_weight(D, n, want_form):
+    """Keys whose scores overflow to -inf (masked by the caller), in the first tile, alone in a whole tile and scattered:
+    weight 0, as the oracle has it for scores of -10^38."""
+    S = 640
+    g = torch.Generator().manual_seed(D + 3)
+    q, k, v = (torch.randn(2, S, D, generator=g).bfloat16() for _ in range(3))
+    q[..., 0] = 4.0
+    k[..., 0] = 0.0
+    masked = list(range(3, 60)) + list(range(256, 384)) + list(range(400, 640, 7))
+    k[:, masked] = 0.0
+    k[:, masked, 0] = -3e38                                             # 4 x -3e38: -inf in 32 bits
+    out, out_f32, row_m, row_d, restarts = _run(q, k, v, n, want_form, False)
+    ref, (want, want_m, want_d) = _oracle(q, k, v, False)
+    gate_attention(out_f32.numpy(), ref, what=f"masked keys D={D} {want_form}")
+    clear = (ref.row_margin >= EPS_REL).reshape(want_m.shape)
+    assert np.array_equal(row_m.numpy()[clear], want_m[clear])
+
+
+@pytest.mark.parametrize("D,n,want_form", FORMS)
+def test_an_infinite_score_spoils_its_own_row_only(D, n, want_form):
+    """A query row with an infinity has scores of +inf and -inf: its max is +inf from the first tile on, its output NaN; no
+    other row, max or restart count notices."""
+    S = 512
+    g = torch.Generator().manual_seed(D + 4)
+    q, k, v = (torch.randn(2, S, D, generator=g).bfloat16() for _ in range(3))
+    k[:, 7::100] *= 8
+    rows = [0, 133, S - 2]
+    q[:, rows] = 0.0
+    plain = _run(q, k, v, n, want_form, False)
+    q[:, rows, 3] = float("inf")
+    got = _run(q, k, v, n, want_form, False)
+    others = [r for r in range(S) if r not in rows]
+    for a, b in zip(plain[:4], got[:4]):
+        assert torch.equal(a[:, others], b[:, others])
+    assert torch.equal(plain[4], got[4]) and int(got[4].sum()) > 0
+    assert torch.isnan(got[1][:, rows]).all() and (got[2][:, rows] == float("inf")).all()
+
+
+@pytest.mark.parametrize("n,want_form", [(1, "one tile"), (80, "two tiles")])
+def test_8_bit_rows_of_nan(n, want_form):
+    """The same with E4M3 Q and K, whose score scale changes with the tile: a query row that holds the NaN code."""
+    S, H = 512, 2
+    assert form(128, H * n, S // 128, False) == want_form
+    g = torch.Generator().manual_seed(5)
+    q, k, v = (torch.randn(1, H, S, 128, generator=g) for _ in range(3))
+    k[:, :, 7::100] *= 8
+    q[:, :, 200] = 0.0
+    (q8, qs, _), (k8, ks, _) = (workloads.quantize_e4m3_tiles(t) for t in (q, k))
+
+    def run():
+        st = binding.baps_attention_fwd_fp8(*(t.cuda().repeat(n, *[1] * (t.dim() - 1)) for t in (q8, k8, v.bfloat16(), qs, ks)),
+                                            causal=False)
+        binding.poll_async_error()
+        return [t[n // 2].cpu() for t in (st.out_f32, st.row_d, st.row_m, st.restarts)]
+    plain = run()
+    q8[:, :, 200, 9] = 0x7F
+    got = run()
+    others = [r for r in range(S) if r != 200]
+    for a, b in zip(plain[:3], got[:3]):
+        assert torch.equal(a[:, others], b[:, others])
+    assert torch.equal(plain[3], got[3]) and int(got[3].sum()) > 0
+    assert torch.isnan(got[0][:, 200]).all() and (got[2][:, 200] == -float("inf")).all()
