@@ -9,56 +9,59 @@
 
 namespace baps {
 
-// One query tile per CTA or two?  Two share the K / V stream and the set-up of the CTA, and one of them works while the
-// other waits (a task, one score tile, takes 1.08 us of a CTA with two against 1.7 of a CTA with one); one halves the
-// chain of tasks that the longest CTA walks through, which is what a grid that does not fill the SMs several times over
-// takes.  Estimate of both in units of a two-tile task, SMs filled longest CTA first: the longest CTA or the average load of
-// an SM, whichever is larger (all CTAs of a bidirectional problem are equally long: whole waves).  Besides its tasks a
-// CTA costs kFixedTwo / kFixedOne (set-up, first scores, epilogues).  The constants are the middle of those that choose the
-// faster form at all of 52 sizes from 4 x 512 to 4 x 32768 (heads x tokens, D = 128).  Measured, one tile / two tiles,
-// causal: 16 x 512 10.0 / 13.8 us, 32 x 1024 22.6 / 24.7, 16 x 2048 33.6 / 43.3, 8 x 4096 57.0 / 79.1, 1 x 16384 219 / 274; and where
-// two are taken: 64 x 512 17.5 / 15.4, 24 x 2048 51.8 / 44.0, 12 x 4096 89.8 / 78.4, 8 x 8192 206 / 145, 2 x 32768 788 / 523;
-// bidirectional 16 x 512 10.8 / 14.8, 8 x 2048 31.3 / 42.4, and 24 x 2048 90.3 / 83.9, 12 x 4096 169 / 154.
+// One query tile per CTA or two (D = 128)?  Two share the K / V stream and the set-up of the CTA, and one of them works
+// while the other waits: a task, one score tile, takes 1.06 us of a CTA with two against 1.68 of a CTA with one
+// (kTaskOne, their ratio).  One halves the chain of tasks that the longest CTA walks through, which is what a grid that does
+// not fill the SMs several times over takes; a single wave of them is always the faster.
+//   All CTAs of a bidirectional problem are equally long: whole waves of them, with two tasks' time for set-up, first scores
+// and epilogue beside the tasks.
+//   Causal: by the load of an SM, all tasks spread evenly, in chains of the longest query tile.  Short chains change over
+// earlier, since the set-up is a larger part of a CTA and one with two tiles pays it once; an odd number of tiles earlier
+// still.  Up to five tiles whole waves show: two tiles a CTA in a second wave of a few CTAs lose to one tile in two full ones.
+// Line and constants are fitted to which form was faster at 796 causal and as many bidirectional sizes of 1 to 385 heads x 128
+// to 32768 tokens, half of them with 8-bit Q / K (one line serves both); the form chosen is at most 5 % behind the other.
+// Measured, one tile / two tiles, causal (heads x tokens): 16 x 512 9.9 / 13.6 us, 32 x 1024 21.5 / 23.7, 16 x 2048 32.3 / 42.0,
+// 8 x 4096 55.6 / 79.9, 1 x 16384 218 / 270, 75 x 384 14.7 / 18.2; and where two are taken: 48 x 640 17.3 / 14.3, 20 x 2048
+// 44.3 / 42.3, 6 x 8192 165 / 145, 3 x 16384 318 / 281, 2 x 32768 808 / 529; bidirectional 8 x 2048 29.8 / 41.7, and 10 x 2048
+// 58.9 / 45.2, 12 x 4096 169 / 152; 8-bit Q / K, causal: 36 x 1024 22.3 / 23.1, and 6 x 8192 155 / 142.
 inline bool one_tile_per_cta(long long heads, int nq, bool causal, int num_sms)
 {
-    constexpr double kFixedTwo = 4.5, kFixedOne = 4.0, kTaskOne = 1.35;
+    constexpr double kFixed = 2.0, kTaskOne = 1.6;
     const long long ctas2 = heads * ((nq + 1) / 2), ctas1 = heads * nq;
-    const double longest1 = kTaskOne * nq + kFixedOne, longest2 = (causal || nq == 1 ? 2 * nq - 1 : 2 * nq) + kFixedTwo;
-    double t1, t2;
+    if (nq == 1) return false;                             // the same work; paired_attention_tc_kernel's set-up is 2 to 7 % shorter
+    if (ctas1 <= num_sms) return true;
     if (causal) {
-        const double tasks = (double)heads * nq * (nq + 1) / 2;
-        const double load1 = (kTaskOne * tasks + kFixedOne * ctas1) / num_sms, load2 = (tasks + kFixedTwo * ctas2) / num_sms;
-        t1 = load1 > longest1 ? load1 : longest1;
-        t2 = load2 > longest2 ? load2 : longest2;
-    } else {
-        t1 = (double)((ctas1 + num_sms - 1) / num_sms) * longest1;
-        t2 = (double)((ctas2 + num_sms - 1) / num_sms) * longest2;
+        const double load = (double)heads * (nq + 1) / (2.0 * num_sms);
+        return load < 1.24 - (nq % 2 ? 2.4 : 1.6) / nq || (nq <= 5 && ctas2 > num_sms && ctas1 <= 2LL * num_sms);
     }
+    const double t1 = (double)((ctas1 + num_sms - 1) / num_sms) * (kTaskOne * nq + kFixed);
+    const double t2 = (double)((ctas2 + num_sms - 1) / num_sms) * (2 * nq + kFixed);
     return t1 < t2;
 }
 
-// Heads of 64: attention_d64_kernel (two CTAs per SM) or attention_tc_kernel with one query tile per CTA, whose
-// sixteen softmax warps are through with a lone tile sooner (1.25 us a task against 1.76 alone and 2.4 shared,
-// but 1.22 per task and SM)?  The former when the SMs are full: more tiles than SMs (bidirectional: tiles 128
-// 22.8 us against 15.4, 160 24.1 / 28.1, 512 47.8 / 57.4, 4096 330 / 403), or an average load of an SM of 1.3 times
-// the longest causal tile (heads x tokens: 24 x 1024 21.5 / 15.6, 24 x 2048 42.8 / 44.2, 2 x 16384 265 / 162,
-// 64 x 8192 1101 / 1269).
+// Heads of 64: attention_d64_kernel (two CTAs per SM) or attention_tc_kernel with one query tile per CTA, whose sixteen
+// softmax warps are through with a lone tile sooner?  The former when the SMs are full: more tiles than SMs, and causal by the
+// load of an SM as above (short chains earlier, since there the set-up of one CTA runs beside the other).  The kernel chosen
+// is at most 2 % behind the other at 398 causal and as many bidirectional sizes, nq = 1 with nearly as many heads as SMs aside
+// (147 x 128: 5.5 / 4.9 us).  Measured, attention_tc_kernel / attention_d64_kernel, causal (heads x tokens): 24 x 1024 15.0 / 16.2
+// us, 16 x 2048 27.4 / 28.3, 2 x 16384 153 / 172; and where the latter is taken: 64 x 512 14.8 / 12.1, 40 x 1024 25.2 / 19.7,
+// 20 x 2048 36.8 / 33.3, 10 x 4096 58.8 / 55.4; bidirectional 8 x 2048 24.2 / 27.2, and 10 x 2048 47.2 / 41.0.
 inline bool two_ctas_per_sm(long long heads, int nq, bool causal, int num_sms)
 {
-    return causal ? 10 * heads * (nq + 1) >= 26LL * num_sms : heads * nq > num_sms;
+    return heads * nq > num_sms && (!causal || (double)heads * (nq + 1) / (2.0 * num_sms) >= 1.04 - 1.65 / nq);
 }
 
 // The kv heads (of all batches) are worked on in chunks: `wide` chunks of size + 1, then chunks of `size`.
 struct KvChunks { int size, wide; };
 
 // Chunks of kv heads whose K and V take 16 MB or a little more, with CTAs enough in each to keep the SMs evenly busy
-// (causal: three for every one that is resident, heavy and light ones mixed; with fewer 32 x 4096 tokens ran 2 %
-// slower, with four the larger chunks cost 1 to 2 % in L2 misses), all of one size but for one head: the last chunk,
-// too, starts with its longest CTAs, and with only a few heads left over these ran alone at the end.  Measured, all kv
-// heads at once -> chunks of 16 MB and what is left -> even chunks (causal, heads x tokens, inputs not in L2): 16 x 16384
-// 1198 -> 1348 -> 1200 us, 36 / 9 x 8192 717 -> 790 -> 719, 8-bit Q / K 64 / 16 x 8192 1341 -> 1430 -> 1340, D = 64
-// 9 x 16384 632 -> 756 -> 611; and what the chunks are for: 96 x 4096 570 -> 535 -> 524, 512 x 1024 of D = 64,
-// bidirectional, 350 -> 334 -> 334.
+// (causal: three for every one that is resident, heavy and light ones mixed), all of one size but for one head: the last
+// chunk, too, starts with its longest CTAs, and with only a few heads left over these would run alone at the end.  Measured,
+// all kv heads at once -> even chunks, calls back to back (causal, heads x tokens): 96 x 4096 521 -> 454 us, 16 x 16384
+// 1138 -> 1100, 36 / 9 x 8192 664 -> 638, 64 / 16 x 8192 1187 -> 1173 (8-bit Q / K 1060 -> 1055), 32 x 4096 173 -> 170; D = 64:
+// 9 x 16384 518 -> 518, 512 x 1024 bidirectional 305 -> 304.  A lone call that finds none of its inputs in L2 takes the same
+// either way, to 0.5 %.  (With the kernels before these a ragged last chunk cost 10 to 20 % at 16 x 16384, 36 / 9 x 8192 and, D = 64,
+// 9 x 16384; two CTAs for every one that is resident 2 % at 32 x 4096.)
 // kv_bytes: of K and V of one head; per_kv: CTAs per kv head.
 inline KvChunks kv_chunks(long long kv_heads, long long kv_bytes, long long per_kv, bool causal, int num_sms, int ctas_per_sm)
 {
@@ -71,8 +74,7 @@ inline KvChunks kv_chunks(long long kv_heads, long long kv_bytes, long long per_
 
 // Which tile of which head a CTA works on.  The kv heads are taken in chunks whose K and V together stay in L2 while
 // their query tiles pass; within a chunk the heavy (late) query tiles come first and the query heads of one kv
-// head are adjacent.  (Taken all at once, 512 heads x 1024 tokens of D = 64 -- 134 MB of K and V -- were read from
-// HBM again for every query tile.)
+// head are adjacent.
 struct WorkItem { int tile, h, hk, b; };
 BAPS_HD WorkItem work_item(int H, int Hkv, int npairs, KvChunks ch, int idx)
 {

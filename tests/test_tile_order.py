@@ -1,22 +1,29 @@
 """The order in which the CTAs of the fused attention take query tiles and heads (``csrc/baps_tile_order.cuh``,
 compiled here as plain C++): every tile once, chunks of kv heads even, and the SMs as evenly busy as without chunks."""
 import heapq
+import os
 import random
+import re
 
 import pytest
 
-from tile_order import SMS, one_tile_per_cta, tiles
+from paper_2602_02071_b200 import build
+from tile_order import SMS, form, one_tile_per_cta, tiles
+
+RULES = open(os.path.join(build.CSRC, "baps_tile_order.cuh")).read()
 
 
 def makespan(items, nq, pairs, slots):
-    """CTAs handed out in order to whichever slot is free first; costs as in one_tile_per_cta (causal)."""
+    """CTAs handed out in order to whichever slot is free first (causal); costs as measured beside one_tile_per_cta, in
+    tasks of a CTA with two query tiles: kTaskOne a task of a CTA with one, kFixed for either."""
+    fixed, task_one = (float(re.search(n + r" = ([\d.]+)", RULES)[1]) for n in ("kFixed", "kTaskOne"))
     free = [0.0] * slots
     for tile, *_ in items:
         if pairs:
             lone = 2 * tile + 1 == nq
-            cost = 4.5 + (2 * tile + 1) + (0 if lone else 2 * tile + 2)
+            cost = fixed + (2 * tile + 1) + (0 if lone else 2 * tile + 2)
         else:
-            cost = 3.5 + 1.25 * (tile + 1)
+            cost = fixed + task_one * (tile + 1)
         heapq.heapreplace(free, free[0] + cost)
     return max(free)
 
@@ -56,3 +63,18 @@ def test_random_shapes():
         nq, key_bytes = rng.choice([1, 3, 8, 16, 31, 64]), rng.choice([256, 384, 512])
         if B * Hkv * g * nq <= 30000:
             check(B, Hkv * g, Hkv, 128 * nq, key_bytes)
+
+
+@pytest.mark.parametrize("D,causal,few,many", [
+    (128, True, [(16, 512), (32, 1024), (16, 2048), (8, 4096), (3, 8192), (2, 16384), (1, 32768), (75, 384), (74, 256)],
+     [(48, 640), (64, 512), (40, 1024), (20, 2048), (12, 4096), (6, 8192), (3, 16384), (2, 32768), (110, 256), (1, 128)]),
+    (128, False, [(36, 512), (8, 2048), (2, 8192), (75, 384)], [(40, 512), (10, 2048), (3, 8192), (12, 4096)]),
+    (64, True, [(36, 512), (24, 1024), (16, 2048), (8, 4096), (3, 8192), (2, 16384), (1, 32768), (74, 256), (74, 128)],
+     [(48, 512), (40, 1024), (20, 2048), (10, 4096), (6, 8192), (3, 16384), (2, 32768), (110, 256), (200, 128)]),
+    (64, False, [(36, 512), (8, 2048), (2, 8192), (74, 128)], [(40, 512), (10, 2048), (3, 8192), (200, 128)])])
+def test_the_form_that_was_measured_to_be_faster(D, causal, few, many):
+    """Sizes (heads, tokens) on both sides of the line, each at least 2 % faster in the form that is taken for it."""
+    for heads, S in few:
+        assert form(D, heads, S // 128, causal) == "one tile", (heads, S)
+    for heads, S in many:
+        assert form(D, heads, S // 128, causal) != "one tile", (heads, S)
