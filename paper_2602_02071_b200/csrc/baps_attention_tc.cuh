@@ -323,14 +323,15 @@ __device__ __forceinline__ void rescale_columns(uint32_t o_addr, int n, float f)
 // exponents of a packed pair of weights.  O~ is touched only when the max moves and e has passed 61: a move without a
 // restart adds 3 at most, so no weight is multiplied by more than 2^64.  The threads of a row take identical decisions.
 // The max of a row moves a handful of times over all key tiles, so an 8-bit tile first asks whether it does in any
-// row of the warp, and nothing below is worked out where it does not.
+// row of the warp, and nothing below is worked out where it does not (attention_tc_kernel at D = 128 aside).
 struct RowState {
     float m, m_ref, d;
     uint32_t escale;
 
     __device__ __forceinline__ void set_scale() { escale = (uint32_t)(int)(m - m_ref) * 0x00800080u; }
-    // A tile in which some row of the warp has a positive T (um: that of the row's maximum mx) or which is restarted.
-    // Moves m to the max that the tile's T are taken against and returns the max after the tile.
+    // For a tile in which some row of the warp has a positive T (um: that of the row's maximum mx) or which is restarted (in
+    // any other it does no more than a rebase that is due).  Moves m to the max that the tile's T are taken against and
+    // returns the max after the tile.
     template <class Rebase>
     __device__ __forceinline__ float decide(float mx, float c, float um, bool restart_tile, Rebase rebase)
     {
@@ -678,6 +679,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
         const float c_base = p.c;
         constexpr bool exact = kMode == BAPS_MODE_EXACT;
         constexpr bool e2e = kMode == BAPS_MODE_E2E_HIF8;
+        // With 128 columns of O~ the branch around the decisions costs more than it saves here, where every warp waits for
+        // the slowest of sixteen (1 x 32768 425 -> 420 us without it, 8-bit Q / K 398 -> 384, B0 = {first, last}, 32 x 4096
+        // bidirectional, 479 -> 474); at D = 64 it is the other way round (306 -> 294 with it).
+        constexpr bool kAlwaysDecide = D == 128;
         const bool count_restarts = p.restarts != nullptr && warp == 0;
         const float over_thr = restart_threshold(p.lambda);
         // per query tile t; O~ and d are rebased past an exponent of 8 in the exact mode, whose factors are not exact
@@ -738,7 +743,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
                 const float um = fmaf(mx, c, -st[T].m);
                 changed = restart_tile || __any_sync(0xffffffffu, um > 0.f);
                 m_next = st[T].m;
-                if (changed) {
+                if (kAlwaysDecide || changed) {
                     if (count_restarts && restart_tile) ++n_restart[T];
                     m_next = st[T].decide(mx, c, um, restart_tile, rebase);
                 }
@@ -813,7 +818,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
             tc_fence_before_sync();
             mbar_arrive(bar(BP + (k & 1)));       // P is in place: the tensor core's burst may go
             st[T].add(sum);
-            if (changed || (kB0Last && hp)) st[T].move(m_next);
+            if ((e2e && kAlwaysDecide) || changed || (kB0Last && hp)) st[T].move(m_next);
             // the next task's scores travel into registers while the loop turns around
             if (has_next) load_scores(k + 1);
             ++k;
