@@ -57,5 +57,11 @@ def test_the_paired_kernel_keeps_the_rules_too():
     assert "await_previous_kernel(" in body and "allow_next_kernel()" in body
     # every role that touches caller memory, or starts a bounded wait, stands behind the wait for the kernel ahead: the
     # producer before its first load (ahead of the CTA-wide barrier that all other roles pass), the softmax warps at entry
-    assert body.index("await_previous_kernel()") < body.index("tma_load_2d(sbase + L::kQOff") < body.index("__syncthreads()")
+    assert body.count("await_previous_kernel()") == 2
+    producer, softmax = (m.start() for m in re.finditer(r"await_previous_kernel\(\)", body))
+    assert producer < body.index("tma_load_2d(sbase + L::kQOff") < body.index("__syncthreads()")
+    # (caller memory beside the tensor maps' is only touched by the softmax warps: the scales, outputs and statistics)
+    touches = [m.start() for m in re.finditer(r"ldg_f32\(|p\.(?:q_scale|k_scale|out|out_f32|row_m|row_d|restarts)\b", body)]
+    assert len(touches) >= 10 and body.index("setmaxnreg.inc") < softmax < min(touches)
+    assert body.count("load_kv(l)") == 2 and producer < body.index("load_kv(l)")
     assert "__launch_bounds__(kTcThreads, 1)" in CODE["baps_attention_pair.cuh"]
