@@ -10,6 +10,7 @@ import pytest
 import torch
 
 from paper_2602_02071_b200 import binding, build
+from tile_order import form
 
 pytestmark = pytest.mark.gpu
 
@@ -23,12 +24,14 @@ def wlib(monkeypatch):
     return lib
 
 
-def _attn(H, S, D, causal=True, **kw):
+def _attn(H, S, D, causal=True, want=None, **kw):
+    assert want is None or form(D, H, S // 128, causal) == want
     q, k, v = (torch.randn(1, H, S, D, device="cuda").bfloat16() for _ in range(3))
     return lambda: binding.baps_attention_fwd_ex(q, k, v, causal=causal, block_q=128, block_k=128, **kw).out_f32
 
 
-def _fp8(H, S):
+def _fp8(H, S, want):
+    assert form(128, H, S // 128, True) == want
     q, k, v = (torch.randn(1, H, S, 128, device="cuda") for _ in range(3))
     q8, k8 = (t.to(torch.float8_e4m3fn) for t in (q, k))
     sc = torch.ones(1, H, S // 128, device="cuda")
@@ -41,14 +44,14 @@ def _rows(cols):
 
 
 @pytest.mark.parametrize("make", [
-    lambda: _attn(2, 512, 128),                                        # one query tile per CTA
-    lambda: _attn(24, 2048, 128),                                      # two query tiles per CTA
-    lambda: _attn(2, 512, 128, mode=binding.MODE_EXACT),               # two, whatever the grid
+    lambda: _attn(2, 512, 128, want="one tile"),
+    lambda: _attn(24, 2048, 128, want="two tiles"),
+    lambda: _attn(2, 512, 128, mode=binding.MODE_EXACT),               # two query tiles per CTA, whatever the grid
     lambda: _attn(2, 512, 128, mode=binding.MODE_EXP2_HIF8),
     lambda: _attn(2, 512, 64, mode=binding.MODE_EXACT),
-    lambda: _attn(2, 512, 64),                                         # heads of 64: one CTA per SM
-    lambda: _attn(64, 1024, 64, causal=False),                         # two
-    lambda: _fp8(24, 2048), lambda: _rows(16384), lambda: _rows(65536)])
+    lambda: _attn(2, 512, 64, want="one tile"),
+    lambda: _attn(64, 1024, 64, causal=False, want="two CTAs per SM"),
+    lambda: _fp8(24, 2048, "two tiles"), lambda: _fp8(2, 512, "one tile"), lambda: _rows(16384), lambda: _rows(65536)])
 def test_waits_start_when_the_kernel_ahead_has_ended(wlib, make):
     call = make()
     want = call()
