@@ -194,9 +194,8 @@ baps_status baps_attention_restart_rates(const void *q, const void *k, const voi
  *   - Limit: B * H * S / 128 <= BAPS_STATIC_SCRATCH_ENTRIES (262144 counters, 1 MiB per GPU that
  *     loads the library, held until the process exits).  Larger problems are refused with
  *     BAPS_ERR_SCRATCH_LIMIT; nothing is launched in that case.
- *   - The first call on a device looks up the device address of the array and, like the other
- *     attention entry points, builds the weight table; that first call synchronises the stream
- *     and should be made before any stream capture is started.
+ *   - The first call on a device looks up the device address of the array and should be made before
+ *     any stream capture is started.
  *   - All calls on a device share the one array.  Every counter the reduction reads is rewritten
  *     by the attention kernel of the same call, so nothing has to be cleared between calls, but two
  *     calls whose kernels overlap on the GPU (different streams) race on it: serialise them.

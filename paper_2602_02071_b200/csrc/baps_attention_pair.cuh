@@ -1,10 +1,11 @@
 // Fused BAPS attention forward for heads of 128 (Algorithm 1, bf16 V, bf16 or 8-bit Q / K), two streams per CTA.
 //
 // One CTA owns two consecutive 128-row query tiles (t = 0, 1) of one (batch, head), which share the K / V stream, and
-// eight softmax warps work on each.  The two streams meet nowhere but in the tensor core: while one waits for its
-// P V and its next Q K^T, or stands at the barrier of its tile-wide vote, the other issues.  A row is shared by two
-// threads (64 columns each), so that what is done once per row and tile -- maxima, vote, decisions, waits, stores --
-// costs half as many instructions per score as with four.
+// eight softmax warps work on each.  The softmax warps of the two streams share no barrier: while one stream waits for its
+// P V and its next Q K^T, or stands at the barrier of its tile-wide vote, the other issues.  They meet at the MMA warp, which
+// serves them in a fixed order, tile by tile: it waits for stream 0's weights even if stream 1's are there first, so that
+// neither gets more than a tile ahead of the other.  A row is shared by two threads (64 columns each), so that what is done
+// once per row and tile -- maxima, vote, decisions, waits, stores -- costs half as many instructions per score as with four.
 //   warps 0-15  softmax: stream t = w / 8; warp w owns rows 32 (w % 4) .. + 31 and the 64 key columns of half
 //               (w / 4) % 2, in two chunks of 32.  Maxima of both chunks, exchange and vote, then the weights of the
 //               second chunk (still in registers) and of the first (read again)
@@ -18,13 +19,16 @@
 // The arithmetic, the bounded waits and the way every role ends after an expired wait are those of
 // attention_tc_kernel; only the row sum is added up in another order (two partial sums per row, not four).
 //
-// What bounds it: the chain of a stream, not a pipe.  A stream takes 3900 cycles per tile (two tiles per SM in that
-// time; the tensor core needs 1024 for one): from its scores to its weights 2500, with two warps per scheduler and
-// stream that do not cover the latency of the lookups, then P V and Q K^T.  Measured against sixteen warps on one tile
-// after the other (attention_tc_kernel with two query tiles; causal, heads x tokens): 8 / 2 x 16384 614 -> 539 us,
-// 64 / 16 x 8192 1250 -> 1092, 64 / 16 x 2048 116 -> 111; bidirectional 128 / 32 x 2048 354 -> 317.  Of that, at the first
-// of these, P V in two halves 559 -> 540, both chunks requested at once 559 -> 538, the two together 539.  The lookups
-// of 32 columns have to be in flight together: sixteen at a time in a rolled loop took 609 to 641.
+// What bounds it: the chain of a stream, not a pipe.  By clock64 stamps (8 / 2 heads x 16384, causal) a stream takes 3980
+// cycles per tile, two tiles per SM in that time, of which the tensor core needs 1024 for each: from its scores to its last
+// weights 2670, with two warps per scheduler and stream that do not cover the latency of the lookups, then P V and Q K^T.
+// The weights of the second chunks are there 500 cycles before the MMA warp, which is still issuing for the other stream,
+// gets to them.  Measured against sixteen warps on one tile after the other (attention_tc_kernel with two query tiles; causal,
+// heads x tokens): 8 / 2 x 16384 614 -> 539 us, 64 / 16 x 8192 1250 -> 1092, 64 / 16 x 2048 116 -> 111; bidirectional 128 / 32 x 2048
+// 354 -> 317.  Of that, at the first of these, P V in two halves 559 -> 540, both chunks requested at once 559 -> 538, the two
+// together 539.  The lookups of 32 columns have to be in flight together: sixteen at a time in a rolled loop took 609 to 641.
+// (tile() and the epilogue are attention_d64_kernel's with other offsets, and P in its score columns: a change to one is to
+// be looked at in the other.)
 #pragma once
 #include "baps_attention_tc.cuh"
 

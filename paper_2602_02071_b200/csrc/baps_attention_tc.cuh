@@ -439,8 +439,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constan
     // ---- setup --------------------------------------------------------------------------------
     // kEarly (D = 64 or one query tile, where a CTA lives for few tasks): the producer lane initialises the barriers itself and
     // starts the Q tiles and the first ring-full of K / V tiles before the CTA-wide barrier, so that the copies
-    // are on their way while the rest of the CTA is still setting up.  (With two tiles at D = 128 the same
-    // change made the steady state 2 % slower, so that path keeps the plain order.)
+    // are on their way while the rest of the CTA is still setting up.  (Two tiles at D = 128, by now the exact and Exp2
+    // modes, keep the plain order: Algorithm 1's steady state was 2 % slower the other way while it ran in that form.)
     constexpr bool kEarly = (D == 64) || kOne;
     constexpr int kQkBoxes = kQK8 ? 1 : D / 64;
     constexpr uint32_t kQkTileBytes = kQK8 ? 128 * D : L::kTileBytes;

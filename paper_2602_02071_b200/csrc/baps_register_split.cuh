@@ -14,8 +14,8 @@ constexpr bool split_fits(const RegisterSplit &s, int regs_at_launch)
     return (s.threads - s.many_threads) * s.few + s.many_threads * s.many <= s.threads * regs_at_launch;
 }
 
-// attention_tc_kernel: a warpgroup of producer, MMA issuer and two idle warps, sixteen softmax warps; 96 at launch.
-// attention_d64_kernel: the same with eight; 80 at launch (two CTAs per SM).  Both use their pool exactly.
+// attention_tc_kernel and paired_attention_tc_kernel: a warpgroup of producer, MMA issuer and two idle warps, sixteen softmax
+// warps; 96 at launch.  attention_d64_kernel: the same with eight; 80 at launch (two CTAs per SM).  All use their pool exactly.
 constexpr RegisterSplit kTcSplit = {640, 64, 512, 104};
 constexpr RegisterSplit kD64Split = {384, 32, 256, 104};
 
