@@ -10,7 +10,7 @@
 namespace baps {
 
 // One query tile per CTA or two (D = 128)?  Two share the K / V stream and the set-up of the CTA, and one of them works
-// while the other waits: a task, one score tile, takes 1.06 us of a CTA with two against 1.68 of a CTA with one
+// while the other waits: a task, one score tile, takes 1.06 us of a CTA with two against 1.65 of a CTA with one
 // (kTaskOne, their ratio).  One halves the chain of tasks that the longest CTA walks through, which is what a grid that does
 // not fill the SMs several times over takes; a single wave of them is always the faster.
 //   All CTAs of a bidirectional problem are equally long: whole waves of them, with two tasks' time for set-up, first scores
@@ -20,10 +20,11 @@ namespace baps {
 // still.  Up to five tiles whole waves show: two tiles a CTA in a second wave of a few CTAs lose to one tile in two full ones.
 // Line and constants are fitted to which form was faster at 796 causal and as many bidirectional sizes of 1 to 385 heads x 128
 // to 32768 tokens, half of them with 8-bit Q / K (one line serves both); the form chosen is at most 5 % behind the other.
-// Measured, one tile / two tiles, causal (heads x tokens): 16 x 512 9.9 / 13.6 us, 32 x 1024 21.5 / 23.7, 16 x 2048 32.3 / 42.0,
-// 8 x 4096 55.6 / 79.9, 1 x 16384 218 / 270, 75 x 384 14.7 / 18.2; and where two are taken: 48 x 640 17.3 / 14.3, 20 x 2048
-// 44.3 / 42.3, 6 x 8192 165 / 145, 3 x 16384 318 / 281, 2 x 32768 808 / 529; bidirectional 8 x 2048 29.8 / 41.7, and 10 x 2048
-// 58.9 / 45.2, 12 x 4096 169 / 152; 8-bit Q / K, causal: 36 x 1024 22.3 / 23.1, and 6 x 8192 155 / 142.
+// Measured, one tile / two tiles, causal (heads x tokens): 16 x 512 9.8 / 13.6 us, 32 x 1024 21.4 / 24.1, 16 x 2048 32.2 / 42.3,
+// 8 x 4096 55.2 / 80.7, 1 x 16384 216 / 271, 75 x 384 14.6 / 18.2; and where two are taken: 48 x 640 17.2 / 14.3, 20 x 2048
+// 44.2 / 42.5, 6 x 8192 164 / 146, 3 x 16384 315 / 282, 2 x 32768 776 / 527; bidirectional 8 x 2048 29.6 / 41.7, and 10 x 2048
+// 58.9 / 45.6, 12 x 4096 168 / 153; 8-bit Q / K, causal: 8 x 4096 51.5 / 77.9, and 20 x 2048 42.2 / 41.7, 6 x 8192 153 / 142; the
+// wrong side of the line: 36 x 1024 23.0 / 23.9.
 inline bool one_tile_per_cta(long long heads, int nq, bool causal, int num_sms)
 {
     constexpr double kFixed = 2.0, kTaskOne = 1.6;
@@ -44,8 +45,8 @@ inline bool one_tile_per_cta(long long heads, int nq, bool causal, int num_sms)
 // load of an SM as above (short chains earlier, since there the set-up of one CTA runs beside the other).  The kernel chosen
 // is at most 2 % behind the other at 398 causal and as many bidirectional sizes, nq = 1 with nearly as many heads as SMs aside
 // (147 x 128: 5.5 / 4.9 us).  Measured, attention_tc_kernel / attention_d64_kernel, causal (heads x tokens): 24 x 1024 15.0 / 16.2
-// us, 16 x 2048 27.4 / 28.3, 2 x 16384 153 / 172; and where the latter is taken: 64 x 512 14.8 / 12.1, 40 x 1024 25.2 / 19.7,
-// 20 x 2048 36.8 / 33.3, 10 x 4096 58.8 / 55.4; bidirectional 8 x 2048 24.2 / 27.2, and 10 x 2048 47.2 / 41.0.
+// us, 16 x 2048 27.5 / 28.4, 2 x 16384 153 / 173; and where the latter is taken: 64 x 512 14.8 / 12.0, 40 x 1024 25.3 / 19.7,
+// 20 x 2048 36.8 / 33.3, 10 x 4096 58.9 / 55.4; bidirectional 8 x 2048 24.3 / 27.1, and 10 x 2048 47.4 / 41.0.
 inline bool two_ctas_per_sm(long long heads, int nq, bool causal, int num_sms)
 {
     return heads * nq > num_sms && (!causal || (double)heads * (nq + 1) / (2.0 * num_sms) >= 1.04 - 1.65 / nq);
