@@ -32,17 +32,16 @@ namespace baps {
 // (integer valued, or -inf before block 0) and the block's largest logit xmax (base-2 score
 // xmax * log2(e)), return the new max.  *restart is set when the restart branch was taken.
 // T of the maximum is formed exactly as for every other element (one fused multiply-add).
-// (ceilf + 0: never -0, which ceilf gives for scores in (-1, 0); against that the table key of a logit of exactly 0 would
-// be that of -0, a positive T's.)
+// (The max may be -0, which ceilf gives for scores in (-1, 0).)
 __device__ __forceinline__ float row_block_update(float m, float xmax, bool first, int lambda,
                                                   bool *restart, float *delta)
 {
     *restart = false; *delta = 0.f;
-    if (first) return fmaxf(m, ceilf(xmax * kLog2e) + 0.f);
+    if (first) return fmaxf(m, ceilf(xmax * kLog2e));
     const float u = fmaf(xmax, kLog2e, -m);
     if (u <= 0.f) return m;                     // T8 <= 0: no restart, delta = 0 (the common case)
     const float t8 = hif8_round(u);
-    if (t8 > (float)lambda) { *restart = true; return fmaxf(m, ceilf(xmax * kLog2e) + 0.f); }
+    if (t8 > (float)lambda) { *restart = true; return fmaxf(m, ceilf(xmax * kLog2e)); }
     const float d = fmaxf(0.f, ceilf(t8));
     *delta = d;
     return m + d;
@@ -70,7 +69,8 @@ __device__ __forceinline__ float lanes_max(float mx)
 // (block j, if `mine`; gm: the max before its group, see scan_groups, or NaN) and left in place of the block's maximum
 // and the max before it:
 //   x = (the max the block's T are taken against: after a restart or in block 0 the new one, otherwise the old
-//       one) * 2^-120, the addend of the table key (exact: that max is an integer);
+//       one) * 2^-120, the addend of the table key (exact: that max is an integer; + 0, because against -0 the key of
+//       a logit of exactly 0 would be that of -0, a positive T's);
 //   y = the power of two that moves the block's weights to the row's final max; with the old max as the
 //       reference, 2^-delta 2^(m_after - m_final) = 2^(m_before - m_final).
 // Read back with one 8-byte load per vector, the same address in all lanes of a block (three shuffles per
@@ -90,7 +90,7 @@ __device__ __forceinline__ unsigned prepare_blocks(float2 *s_blk, float gm, int 
         bool rs; float dl;
         const float ma = row_block_update(b.y, b.x, first, lambda, &rs, &dl);
         const float mref = (first || rs) ? ma : b.y;
-        s_blk[j] = make_float2(mref * kTiny, exp2f(mref - mfinal));
+        s_blk[j] = make_float2(fmaf(mref, kTiny, 0.f), exp2f(mref - mfinal));
         if (CODES) block_exp[j] = (int)(mref - mfinal);
         pos = (CODES || !first) && fmaf(b.x, kLog2e, -mref) > 0.f;
     }

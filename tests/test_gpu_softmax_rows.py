@@ -183,14 +183,15 @@ def test_softmax_rows_any_length(chunks, block_k):
 
 
 @pytest.mark.parametrize("first", [[-0.3], [-4.0, -0.3]])
-@pytest.mark.parametrize("cols", [640, 1024, 3200, 8192, 12800, 32768, 49152, 65536])
+@pytest.mark.parametrize("cols", [640, 1024, 2048, 3200, 4096, 8192, 12800, 16384, 32768, 49152, 65536])
 def test_softmax_rows_max_that_rounds_up_to_zero(cols, first):
     """The largest base-2 logit so far lies in (-1, 0), in block 0 or after a restart, so that the max is zero; all later
     logits are zero exactly (padding): T = 0, weight 1.  Every kernel, both outputs."""
     x = torch.zeros(3, cols)
     x[:, :128 * len(first)] = torch.tensor(first).repeat_interleave(128)
-    got = binding.baps_softmax_rows(x.cuda(), block_k=128).cpu().numpy()
-    want = oracle.softmax_rows(x.numpy(), block_k=128)
-    # weights are table entries or fp32 powers of two: what is left is the fp32 sum and the last two roundings
-    assert np.allclose(got, want, rtol=2e-6, atol=0)
-    _check_codes(x, 128, f"zero max cols={cols}")
+    for bk in (128, 64):
+        got = binding.baps_softmax_rows(x.cuda(), block_k=bk).cpu().numpy()
+        want = oracle.softmax_rows(x.numpy(), block_k=bk)
+        # weights are table entries or fp32 powers of two: what is left is the fp32 sum and the last two roundings
+        assert np.allclose(got, want, rtol=2e-6, atol=0)
+        _check_codes(x, bk, f"zero max cols={cols} bk={bk}")
